@@ -199,7 +199,7 @@ def job_value(voxels_per_rank, world_size, ms_per_step_max):
 
 def kernel_sources_sha():
     h = hashlib.sha256()
-    for f in ("pfc_fused.cu", "pfc_fused_kernel.cuh", "pfc_fused_sym.cu", "pfc_device.cuh", "pfc_internal.h"):
+    for f in ("pfc_pair_kernel.cuh", "pfc_pair.cuh", "pfc_pair_sym.cu", "pfc_device.cuh", "pfc_internal.h"):
         with open(os.path.join(ROOT, "paper_2103_04856_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -340,11 +340,7 @@ def membrane_block(pfc, I, flush, steps, peak, peak_kind, with_cpu):
     acc1 = accuracy(pfc, [inst], cur)
     del A, B, cur
     peaks, hk = load_peaks()
-    # a batch's automatic tile height (pfc_batch_create): 16 or 13 rows by padded rows times the
-    # measured cost of a row (the general 16-row batched sweep's rows cost 4 % more)
-    ny = inst.shape[1]
-    ty = 13 if ((ny + 12) // 13 * 13) < ((ny + 15) // 16 * 16) * 1.04 else 16
-    roof = alu_roofline(workload_flops([inst]), msw, peak, peak_kind, f"k_fused<float,{ty},STEP,64> (general sweep)")
+    roof = alu_roofline(workload_flops([inst]), msw, peak, peak_kind, "k_pair<20,STEP,64> (general sweep)")
     hbm = 8.0 * vox / (msw * 1e-3) / 1e9
     roof["traffic"] = None
     roof["traffic_note"] = "no ncu capture of this launch (512^3 is above the capture size rule)"
@@ -906,7 +902,7 @@ def main():
     # 185-211 flop per 8 B is ~2x GB300's FP32/HBM balance: the sweep is bound
     # by arithmetic issue, not by HBM; the HBM fraction is reported beside it
     roofline = alu_roofline(flops_launch, ms_sweep, fp32_peak, fp32_kind,
-                            f"k_fused<float,{ty_used},STEP,64{',SYM' if all_sym else ''}> (batched fused sweep)")
+                            f"k_pair<STEP,64{',SYM' if all_sym else ''}> (batched fused sweep, tile_y {ty_used})")
     roofline.update({"traffic": traffic, "derived_peak": FP32_PEAK_TFLOPS,
                      "derived_peak_kind": "152 SM x 128 FP32 lanes x 2 flop x 2070 MHz",
                      "flops_per_voxel_step": flops_launch / vox, "voxels_per_launch": vox,

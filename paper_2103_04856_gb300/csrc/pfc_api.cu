@@ -113,43 +113,11 @@ static pfc_status check_problem(const pfc_problem* p)
     return PFC_OK;
 }
 
-// Automatic tile height of a batch (its launches run the batched
-// instantiations, MAXI = 64): the one of 16 and 13 rows with the smaller
-// cost, the rows padded to whole tiles (summed over the problems' x-z planes)
-// times the measured cost of a row.  In the symmetric sweep a 13-row tile's
-// row costs 4.3 % more (four 128^3 problems: 87.5 us at 16 rows, 92.7 us at
-// 13, padded to 130 rows).  In the general sweep the 16-row instantiation (20
-// warps at 96 registers) keeps more values in local memory than the 13-row
-// one (16 warps at 128 registers), the more so when the problems' coefficients
-// differ (they are then loaded per use from the descriptor table): its row
-// costs 3.5 % more with one coefficient set (a 512^3 problem: 1.795 ms at 16
-// rows, 1.761 ms at 13, padded to 520 rows) and 10 % more with many (the
-// 64-instance mixed batch of 64^3, 96^3 and 128^3 problems: 1.03 against 0.97
-// ms per step, 4.1 % more rows at 13).  Single problems (MAXI = 1) take
-// default_tile_y.
-static int auto_tile_y(const pfc_problem* p, int n)
-{
-    if (p[0].prec == PFC_FP64) return 8;
-    bool general = false, one_set = true;
-    double rows16 = 0.0, rows13 = 0.0;
-    for (int k = 0; k < n; ++k) {
-        const double plane = (double)p[k].nx * p[k].nz;
-        rows16 += plane * ((p[k].ny + 15) / 16 * 16);
-        rows13 += plane * ((p[k].ny + 12) / 13 * 13);
-        general = general || !make_coef<float>(p[k].a, p[k].h, p[k].eps, p[k].xi, p[k].well).sym;
-        one_set = one_set && memcmp(p[k].a, p[0].a, sizeof(p[0].a)) == 0 && p[k].h == p[0].h &&
-                  p[k].eps == p[0].eps && p[k].xi == p[0].xi && p[k].well == p[0].well;
-    }
-    const double c16 = general ? (one_set ? 1.035 : 1.10) : 1.0, c13 = general ? 1.0 : 1.043;
-    return rows13 * c13 < rows16 * c16 ? 13 : 16;
-}
-
 // Launch geometry of one problem: 32 x tile_y columns per CTA, z chunks chosen
 // so that the grid fills the GPU about twice unless the user fixed tile_z.
 static void geometry(const pfc_problem* p, int sms, int* tile_y, int* zc, int* tx, int* ty, int* cz)
 {
-    const bool general = !make_coef<float>(p->a, p->h, p->eps, p->xi, p->well).sym;
-    int tyv = p->tile_y ? p->tile_y : default_tile_y(p->ny, p->prec == PFC_FP64, general);
+    int tyv = p->tile_y ? p->tile_y : default_tile_y(p->ny, p->prec == PFC_FP64);
     *tile_y = tyv;
     *tx = (p->nx + 31) / 32;
     *ty = (p->ny + tyv - 1) / tyv;
@@ -235,7 +203,7 @@ extern "C" pfc_status pfc_create(const pfc_problem* prob, pfc_ctx** out)
         return fail(PFC_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
     }
     geometry(prob, device_sms(), &c->tile_y, &c->zc, &c->tiles_x, &c->tiles_y, &c->chunks_z);
-    c->nblocks = (int)fused_slots(prob->nx, prob->ny, prob->nz, c->tile_y, prob->tile_z);
+    c->nblocks = (int)fused_grid(fused_units(prob->nx, prob->ny, prob->nz), prob->tile_z);
     c->plain_nblocks = plain_blocks(c->N);
     const int nparts = c->nblocks > c->plain_nblocks ? c->nblocks : c->plain_nblocks;
     bool ok = cudaMalloc(&c->ping, (size_t)c->esz * c->N) == cudaSuccess &&
@@ -686,7 +654,7 @@ extern "C" pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32
     local.nz = nz_local;
     int zc, tx, ty, cz;
     geometry(&local, device_sms(), &sl->tile_y, &zc, &tx, &ty, &cz);
-    sl->nblocks = (int)fused_slots(prob->nx, prob->ny, nz_local, sl->tile_y, prob->tile_z);
+    sl->nblocks = (int)fused_grid(fused_units(prob->nx, prob->ny, nz_local), prob->tile_z);
     const size_t bytes = sizeof(double) * ((size_t)NPART * sl->nblocks + NSCAL) + sizeof(unsigned) * NINTS;
     if (cudaMalloc((void**)&sl->mem, bytes) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -876,7 +844,7 @@ extern "C" pfc_status pfc_batch_create(const pfc_problem* probs, int32_t n, pfc_
     b->host.resize(n);
     b->ping.assign(n, nullptr);
     bool ok = true;
-    b->tile_y = probs[0].tile_y ? probs[0].tile_y : auto_tile_y(probs, n);   // one height for all instances
+    b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(probs[0].ny, false);   // one height for all instances
     b->max_run = probs[0].tile_z;
     long long units = 0;
     for (int k = 0; k < n && ok; ++k) {
@@ -889,7 +857,7 @@ extern "C" pfc_status pfc_batch_create(const pfc_problem* probs, int32_t n, pfc_
         in.nx = p.nx; in.ny = p.ny; in.nz = p.nz;
         in.zc = zc;
         in.tiles_x = tx; in.tiles_y = tyn; in.chunks_z = cz;
-        units += (long long)tx * tyn * p.nz;
+        units += fused_units(p.nx, p.ny, p.nz);
         in.C = make_coef<float>(p.a, p.h, p.eps, p.xi, p.well, 0.0, nullptr, 0, refine_of(p));
         in.inv_N = 1.0 / ((double)p.nx * p.ny * p.nz);
         ok = cudaMalloc(&b->ping[k], sizeof(float) * (size_t)p.nx * p.ny * p.nz) == cudaSuccess;

@@ -108,31 +108,32 @@ __device__ __forceinline__ DF df_div(DF a, DF b)
 }
 
 // D of eq. Meps's M in double-float from the 19 raw stencil values of the
-// voxel (exact floats in three u planes: pm, p0, pp point at the voxel,
-// `pitch` is the row pitch) plus the offset c the loads add: differences
+// voxel (exact floats in three u planes: pm, p0, pp point at the voxel; xs is
+// the element distance to x + 1, yu and yd the offsets of y + 1 and y - 1)
+// plus the offset c the loads add: differences
 // of the inputs are exact (two-sum), every later operation keeps about 44
 // bits, so the cancellation in 2S - T^2 no longer loses the result.  Kept out
 // of line: it runs for few voxels and must not add registers to the float
 // hot path.
 template <typename T>
-__device__ __noinline__ T discriminant_df_at(const CoefD& R, int well, const T* pm, const T* p0, const T* pp, int pitch,
-                                             double c)
+__device__ __noinline__ T discriminant_df_at(const CoefD& R, int well, const T* pm, const T* p0, const T* pp, int xs,
+                                             int yu, int yd, double c)
 {
     const float ch = (float)c;
     const DF cdf = { ch, (float)(c - (double)ch) };
     const float uc = (float)p0[0];
     const DF u0 = df_add(DF{ uc, 0.0f }, cdf);
     auto f = [](T v) { return (float)v; };
-    auto diff = [&](const T* p, int o) { return df_two_sum(f(p[o]), -f(p[-o])); };                  // u(+) - u(-)
-    auto lap = [&](const T* p, int o) { return df_sub(df_two_sum(f(p[o]), f(p[-o])), DF{ 2.0f * uc, 0.0f }); };
+    auto diff = [&](const T* p, int op, int om) { return df_two_sum(f(p[op]), -f(p[om])); };        // u(+) - u(-)
+    auto lap = [&](const T* p, int op, int om) { return df_sub(df_two_sum(f(p[op]), f(p[om])), DF{ 2.0f * uc, 0.0f }); };
     const DF kd = { R.kd_h, R.kd_l }, ko = { R.ko_h, R.ko_l }, sg = { R.sg_h, R.sg_l };
-    const DF Gx = df_mul(diff(p0, 1), sg), Gy = df_mul(diff(p0, pitch), sg);
+    const DF Gx = df_mul(diff(p0, xs, -xs), sg), Gy = df_mul(diff(p0, yu, yd), sg);
     const DF Gz = df_mul(df_two_sum(f(pp[0]), -f(pm[0])), sg);
-    const DF hxx = lap(p0, 1), hyy = lap(p0, pitch);
+    const DF hxx = lap(p0, xs, -xs), hyy = lap(p0, yu, yd);
     const DF hzz = df_sub(df_two_sum(f(pp[0]), f(pm[0])), DF{ 2.0f * uc, 0.0f });
-    const DF hxy = df_sub(df_two_sum(f(p0[pitch + 1]), -f(p0[pitch - 1])), df_two_sum(f(p0[-pitch + 1]), -f(p0[-pitch - 1])));
-    const DF hxz = df_sub(df_two_sum(f(pp[1]), -f(pp[-1])), df_two_sum(f(pm[1]), -f(pm[-1])));
-    const DF hyz = df_sub(df_two_sum(f(pp[pitch]), -f(pp[-pitch])), df_two_sum(f(pm[pitch]), -f(pm[-pitch])));
+    const DF hxy = df_sub(df_two_sum(f(p0[yu + xs]), -f(p0[yu - xs])), df_two_sum(f(p0[yd + xs]), -f(p0[yd - xs])));
+    const DF hxz = df_sub(df_two_sum(f(pp[xs]), -f(pp[-xs])), df_two_sum(f(pm[xs]), -f(pm[-xs])));
+    const DF hyz = df_sub(df_two_sum(f(pp[yu]), -f(pp[yd])), df_two_sum(f(pm[yu]), -f(pm[yd])));
     const DF rho = df_add(df_add(df_mul(Gx, Gx), df_mul(Gy, Gy)), df_add(df_mul(Gz, Gz), DF{ R.xi2_h, R.xi2_l }));
     DF w;   // W'(u) / eps
     const DF one = { 1.0f, 0.0f };
@@ -228,11 +229,7 @@ struct refines<NoRefine> {
 // a3 r, c3 r and c5 r, which stay exact zeros with r = r' = 0; D, P and
 // sqrt(P) are then not computed, with the same result bits.
 //
-// RAWD: ct.dx, ct.dy, ct.dz are returned without the stencil scale sg =
-// 1/(2h) (the caller folds it into the FMAs that combine them with the
-// second-difference cotangents).
-template <typename T, bool GRAD, bool ORIENT = false, bool PROJ = false, bool SKIPD = false, bool RAWD = false,
-          class Refine = NoRefine>
+template <typename T, bool GRAD, bool ORIENT = false, bool PROJ = false, bool SKIPD = false, class Refine = NoRefine>
 __device__ __forceinline__ T voxel_eval(const Coef<T>& C, T u0, T dx, T dy, T dz, T hxx, T hyy,
                                         T hzz, T hxy, T hxz, T hyz, Cot<T>& ct, const Refine& refine = Refine())
 {
@@ -362,11 +359,11 @@ __device__ __forceinline__ T voxel_eval(const Coef<T>& C, T u0, T dx, T dy, T dz
         const T al = -T(2) * irho;
         const T be = fma_(T(2) * GBG * irho, irho, fma_(dq, iq, C.c6x2));
         ct.u = T(0);
-        ct.dx = RAWD ? fma_(al, BGx, be * Gx) : C.sg * fma_(al, BGx, be * Gx);
-        ct.dy = RAWD ? fma_(al, BGy, be * Gy) : C.sg * fma_(al, BGy, be * Gy);
-        ct.dz = RAWD ? fma_(al, BGz, be * Gz) : C.sg * fma_(al, BGz, be * Gz);
+        ct.dx = C.sg * fma_(al, BGx, be * Gx);
+        ct.dy = C.sg * fma_(al, BGy, be * Gy);
+        ct.dz = C.sg * fma_(al, BGz, be * Gz);
         if (ORIENT) {
-            const T ot = RAWD ? T(2) * C.c7 * tg : T(2) * C.c7 * tg * C.sg;
+            const T ot = T(2) * C.c7 * tg * C.sg;
             ct.dx = fma_(ot, C.th0, ct.dx);
             ct.dy = fma_(ot, C.th1, ct.dy);
             ct.dz = fma_(ot, C.th2, ct.dz);
@@ -382,11 +379,11 @@ __device__ __forceinline__ T voxel_eval(const Coef<T>& C, T u0, T dx, T dy, T dz
     ct.u = wpp * C.inv_eps * GLG * irho;
     const T al = T(2) * wr;
     const T be = fma_(-al * GLG, irho, fma_(dq, iq, C.c6x2));
-    ct.dx = RAWD ? fma_(al, LGx, be * Gx) : C.sg * fma_(al, LGx, be * Gx);
-    ct.dy = RAWD ? fma_(al, LGy, be * Gy) : C.sg * fma_(al, LGy, be * Gy);
-    ct.dz = RAWD ? fma_(al, LGz, be * Gz) : C.sg * fma_(al, LGz, be * Gz);
+    ct.dx = C.sg * fma_(al, LGx, be * Gx);
+    ct.dy = C.sg * fma_(al, LGy, be * Gy);
+    ct.dz = C.sg * fma_(al, LGz, be * Gz);
     if (ORIENT) {
-        const T ot = RAWD ? T(2) * C.c7 * tg : T(2) * C.c7 * tg * C.sg;
+        const T ot = T(2) * C.c7 * tg * C.sg;
         ct.dx = fma_(ot, C.th0, ct.dx);
         ct.dy = fma_(ot, C.th1, ct.dy);
         ct.dz = fma_(ot, C.th2, ct.dz);

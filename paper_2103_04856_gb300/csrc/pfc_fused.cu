@@ -177,6 +177,16 @@ Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, 
     C.sym = (C.c3 == T(0) && C.c5 == T(0)) ? 1 : 0;
     // the refinement test is scale > rthr max(|D|, xi): 2^16 = 2^22 / 2^6, or never
     C.rthr = refine ? T(65536) : T(INFINITY);
+    const double kd = C.R.kd, sg = C.R.sg, K = 1.0 / (eps * kd);
+    C.wA = (T)(well == 0 ? -12.0 * K : 3.0 * K);
+    C.wB = (T)(well == 0 ? 2.0 * K : -K);
+    const double n[5] = { (double)C.c1 * kd * kd, (double)C.c2 * kd * kd, 0.5 * C.c4 * sg * kd, (double)C.c6 * sg * sg,
+                          xi * xi / (sg * sg) };
+    C.n1 = (T)n[0]; C.n2 = (T)n[1]; C.n4 = (T)n[2]; C.n6 = (T)n[3]; C.nx2 = (T)n[4];
+    auto fits = [](double v) { return v == 0.0 || (fabs(v) > 1e-30 && fabs(v) < 1e30); };
+    C.nform = C.sym && n[4] > 1e-30;
+    for (double v : n) C.nform = C.nform && fits(v);
+    C.nform = C.nform && fits(K);
     return C;
 }
 template Coef<float> make_coef<float>(const double*, double, double, double, int, double, const double*, int, int);
@@ -247,12 +257,9 @@ long long fused_grid(long long units, int max_run)
     return G < units ? G : units;
 }
 
-long long fused_slots(int nx, int ny, int nz, int tile_y, int max_run)
+long long fused_units(int nx, int ny, int nz)
 {
-    const long long tx = (nx + TX - 1) / TX;
-    const long long a = fused_grid(tx * ((ny + tile_y - 1) / tile_y) * nz, max_run);
-    const long long b = fused_grid(tx * ((ny + EXT_TILE_Y - 1) / EXT_TILE_Y) * nz, max_run);
-    return a > b ? a : b;
+    return (long long)((nx + TX - 1) / TX) * ((ny + 7) / 8) * nz;
 }
 
 template <typename T, int TY, int EXT = 0>
@@ -262,13 +269,10 @@ static cudaError_t launch_mode(const Inst<T>& in, int mode, int max_run, cudaStr
     L.n = 1;
     L.inst[0] = in;
     plan(L, TY, max_run);
-    if constexpr (EXT == 0 && std::is_same<T, float>::value) {
-        if (in.C.sym) return launch_fused_sym<1>(L, TY, mode, s);
-    }
     switch (mode) {
-    case MODE_ENERGY: return launch_kernel<T, TY, MODE_ENERGY, 1, EXT>(L, L.grid, s);
-    case MODE_GRAD: return launch_kernel<T, TY, MODE_GRAD, 1, EXT>(L, L.grid, s);
-    case MODE_STEP: return launch_kernel<T, TY, MODE_STEP, 1, EXT>(L, L.grid, s);
+    case MODE_ENERGY: return launch_kernel<T, TY, MODE_ENERGY, EXT>(L, L.grid, s);
+    case MODE_GRAD: return launch_kernel<T, TY, MODE_GRAD, EXT>(L, L.grid, s);
+    case MODE_STEP: return launch_kernel<T, TY, MODE_STEP, EXT>(L, L.grid, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -279,25 +283,23 @@ cudaError_t launch_fused(const Inst<T>& in, int mode, int tile_y, int max_run, c
     if (in.halo) return launch_fused_halo<T>(in, mode, tile_y, max_run, s);
     if (in.C.proj) return launch_mode<T, EXT_TILE_Y, 2>(in, mode, max_run, s);
     if (needs_ext(in)) return launch_mode<T, EXT_TILE_Y, 1>(in, mode, max_run, s);
-    if (tile_y == 8) return launch_mode<T, 8>(in, mode, max_run, s);
-    if (tile_y == 13) return launch_mode<T, 13>(in, mode, max_run, s);
-    return launch_mode<T, 16>(in, mode, max_run, s);
+    if constexpr (std::is_same<T, float>::value) {
+        Launch<float, 1> L;
+        L.n = 1;
+        L.inst[0] = in;
+        return in.C.nform ? launch_pair_sym<1>(L, mode, tile_y, max_run, s) : launch_pair<1>(L, mode, tile_y, max_run, s);
+    } else {
+        if (tile_y == 8) return launch_mode<T, 8>(in, mode, max_run, s);
+        if (tile_y == 13) return launch_mode<T, 13>(in, mode, max_run, s);
+        return launch_mode<T, 16>(in, mode, max_run, s);
+    }
 }
 template cudaError_t launch_fused<float>(const Inst<float>&, int, int, int, cudaStream_t);
 template cudaError_t launch_fused<double>(const Inst<double>&, int, int, int, cudaStream_t);
 
 // Batches of up to BATCH_MAX problems go in one launch (their descriptors
 // travel as kernel parameters); larger batches take one launch per group.
-// When every problem of a group has the same coefficients and step size, the
-// launch's per-voxel arithmetic reads them at fixed constant-bank offsets
-// (UNI) instead of loading them from the run's problem descriptor at every
-// use (measured: a 256^3 problem 5 % faster).  Splitting a group with two
-// coefficient sets into two such launches measured 19 % slower on the four
-// 128^3 validation problems (each CTA's runs halve, and a launch gap is
-// added), so only single-set groups take it.
 // MODE_STEP (descent steps) or MODE_GRAD (energies and gradients).
-constexpr int kUniGroups = 1;
-
 cudaError_t launch_fused_batch(const Inst<float>* insts, int n_inst, int tile_y, int max_run, cudaStream_t s,
                                int mode)
 {
@@ -305,48 +307,14 @@ cudaError_t launch_fused_batch(const Inst<float>* insts, int n_inst, int tile_y,
     thread_local Launch<float, BATCH_MAX> L;   // host staging (per thread); the launch copies it
     for (int g0 = 0; g0 < n_inst; g0 += BATCH_MAX) {
         const int cnt = n_inst - g0 < BATCH_MAX ? n_inst - g0 : BATCH_MAX;
-        // sets of equal coefficients (bitwise: make_coef clears the padding) and step size
-        int set[BATCH_MAX], rep[kUniGroups + 1], nsets = 0;
-        bool ext = false;
-        for (int k = 0; k < cnt && nsets <= kUniGroups; ++k) {
-            const Inst<float>& in = insts[g0 + k];
-            ext = ext || needs_ext(in);
-            int j = 0;
-            while (j < nsets && !(memcmp(&insts[g0 + rep[j]].C, &in.C, sizeof(Coef<float>)) == 0 &&
-                                  insts[g0 + rep[j]].tau == in.tau))
-                ++j;
-            if (j == nsets) rep[nsets++] = k;
-            set[k] = j;
-        }
-        if (!ext && nsets <= kUniGroups) {
-            for (int j = 0; j < nsets; ++j) {
-                L.n = 0;
-                for (int k = 0; k < cnt; ++k)
-                    if (set[k] == j) L.inst[L.n++] = insts[g0 + k];
-                L.C0 = insts[g0 + rep[j]].C;
-                L.tau0 = insts[g0 + rep[j]].tau;
-                plan(L, tile_y, max_run);
-                cudaError_t e = launch_fused_uni(L, tile_y, mode, L.C0.sym != 0, s);
-                if (e != cudaSuccess) return e;
-            }
-            continue;
-        }
         L.n = cnt;
-        for (int k = 0; k < cnt; ++k) L.inst[k] = insts[g0 + k];
-        plan(L, tile_y, max_run);
         bool sym = true;
-        for (int k = 0; k < cnt; ++k) sym = sym && L.inst[k].C.sym && !needs_ext(L.inst[k]);
-        cudaError_t e;
-        if (sym)
-            e = launch_fused_sym<BATCH_MAX>(L, tile_y, mode, s);
-        else if (mode == MODE_STEP)
-            e = tile_y == 8    ? launch_kernel<float, 8, MODE_STEP, BATCH_MAX>(L, L.grid, s)
-                : tile_y == 13 ? launch_kernel<float, 13, MODE_STEP, BATCH_MAX>(L, L.grid, s)
-                               : launch_kernel<float, 16, MODE_STEP, BATCH_MAX>(L, L.grid, s);
-        else
-            e = tile_y == 8    ? launch_kernel<float, 8, MODE_GRAD, BATCH_MAX>(L, L.grid, s)
-                : tile_y == 13 ? launch_kernel<float, 13, MODE_GRAD, BATCH_MAX>(L, L.grid, s)
-                               : launch_kernel<float, 16, MODE_GRAD, BATCH_MAX>(L, L.grid, s);
+        for (int k = 0; k < cnt; ++k) {
+            L.inst[k] = insts[g0 + k];
+            sym = sym && L.inst[k].C.nform;
+        }
+        cudaError_t e = sym ? launch_pair_sym<BATCH_MAX>(L, mode, tile_y, max_run, s)
+                            : launch_pair<BATCH_MAX>(L, mode, tile_y, max_run, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -24,10 +24,8 @@
 // coefficients of its column one plane ahead of their use); 2 = the same
 // with the tangent-projected M = -eps P Hess u P.
 //
-// The template and its launch are shared by pfc_fused.cu (every sweep) and
-// pfc_fused_sym.cu (the sweep for polynomials symmetric in kappa1, kappa2,
-// whose sqrt(D+) terms have weight zero), so that the two sets of
-// instantiations compile as separate translation units.
+// FP64 sweeps and the extended ones run here; FP32 without extensions runs two
+// voxels per thread (k_pair, pfc_pair_kernel.cuh).
 #pragma once
 
 #include <type_traits>
@@ -99,20 +97,14 @@ __device__ __forceinline__ void bar_cta() { asm volatile("barrier.sync 0;\n" :::
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// SYM: every problem of the launch has c3 = c5 = 0 (FP32, EXT = 0 only): the
-// sqrt(D+) terms, whose weight is exactly zero then, are not compiled in.
 // HALO: the problem is a z-slab whose planes beyond its ends come from
 // in.halo (instantiated only for slab launches, in pfc_fused_slab.cu: the
 // check costs the other launches registers they do not have).
-// UNI (batched launches, EXT = 0): every problem of the launch has the
-// coefficients L.C0 and the step size L.tau0; per-voxel arithmetic takes them
-// as constant-bank operands, where in.C at the run-time problem index costs a
-// load per use (pfc_fused_uni.cu).
-template <typename T, int TY, int MODE, int MAXI, int EXT = 0, bool SYM = false, bool HALO = false, bool UNI = false>
+template <typename T, int TY, int MODE, int EXT = 0, bool HALO = false>
 __global__ void __launch_bounds__(Tile<TY>::NT, 1)
-k_fused(const __grid_constant__ Launch<T, MAXI> L)
+k_fused(const __grid_constant__ Launch<T, 1> L)
 {
-    static_assert(!SYM || (EXT == 0 && sizeof(T) == 4), "the symmetric sweep is FP32 without extensions");
+    static_assert(EXT != 0 || sizeof(T) == 8, "FP32 without extensions runs k_pair");
     using TL = Tile<TY>;
     constexpr int EX = TL::EX, NEXT = TL::NEXT, NT = TL::NT, UY = TL::UY, PLANE = TL::PLANE;
     constexpr int VEC = 16 / (int)sizeof(T);
@@ -150,34 +142,13 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
     // per-thread sums of the problem being processed, in the arithmetic type
     // (a few hundred terms each), combined in FP64 across threads and CTAs
     T se = 0, su = 0, sg = 0, sag = 0, gmax = 0, sout = 0;
-    int cur = -1;                                 // problem the sums belong to
-    auto flush = [&]() {
-        const T v[NPART] = { se, su, sg, sag, gmax, sout };
-        block_sums<NT>(v, scr, tot);
-        const Inst<T>& pin = L.inst[cur];
-        finish_problem(pin, (int)blockIdx.x - pin.first_block, MODE, tot, MAXI > 1);
-        se = su = sg = sag = gmax = sout = 0;
-    };
-
     // this CTA's share of the work units
     const long long W = L.units;
     long long U = (long long)blockIdx.x * W / L.grid;
     const long long Uend = ((long long)blockIdx.x + 1) * W / L.grid;
+    const Inst<T>& in = L.inst[0];
     while (U < Uend) {
-        // ---- the run: one column tile of one problem, a contiguous z range
-        int k = 0;
-        if (MAXI > 1) {
-            int hi = L.n - 1;
-            while (k < hi) {
-                const int mid = (k + hi + 1) >> 1;
-                if (L.inst[mid].unit_base <= U) k = mid; else hi = mid - 1;
-            }
-        }
-        if (k != cur) {
-            if (cur >= 0) flush();
-            cur = k;
-        }
-        const Inst<T>& in = L.inst[k];
+        // ---- the run: one column tile of the problem, a contiguous z range
         const int nx = in.nx, ny = in.ny, nz = in.nz;
         const long long rel = U - in.unit_base;
         const int ct = (int)(rel / nz);
@@ -189,21 +160,6 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
         const int plast = zend + 1;                    // last u plane needed
         const size_t plane_g = (size_t)nx * ny;
         const int gx = x0 + ex - 1, gy = y0 + ey - 1;
-        const bool interior0 = warp < TY && gx < nx && gy < ny;
-        // batch steps: an instance whose scalars became non-finite in an
-        // earlier step of the chain is retired (the flag is written only by
-        // the finish of a launch, after every CTA has read it): its runs
-        // write NaN and add nothing to its sums
-        if constexpr (MAXI > 1 && MODE == MODE_STEP) {
-            if (__ldcg(&in.ints[I_NONFINITE])) {
-                if (interior0) {
-                    T* o = in.out + (size_t)z0 * plane_g + (size_t)gy * nx + gx;
-                    for (int z = z0; z < zend; ++z, o += plane_g) *o = T(NAN);
-                }
-                continue;
-            }
-        }
-
         using Y = std::true_type;
         using N = std::false_type;
         // The rest of the run, instantiated once for the row warps (ROLE =
@@ -306,7 +262,7 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
                     if (interior) *optr = g;
                 } else {
                     const T u0 = (sizeof(T) == 4 ? umm_ : us[(kz & (NBUF - 1)) * PLANE + uc]) + cin;
-                    const T v = fma_(UNI ? -L.tau0 : -in.tau, g, u0);
+                    const T v = fma_(-in.tau, g, u0);
                     if (interior) *optr = v;
                     su = fma_(wI, u0, su);
                     sout = fma_(wI, v, sout);
@@ -366,7 +322,6 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
                 Cot<T> ctv;
                 const Coef<T>& CC = [&]() -> const Coef<T>& {
                     if constexpr (EXT) return Cv;
-                    else if constexpr (UNI) return L.C0;
                     else return in.C;
                 }();
                 // re-evaluation of D from the exact float inputs (float path only):
@@ -377,33 +332,22 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
                     // c1 .. c6, and a reference to the per-plane copy Cv would put it in
                     // local memory)
                     if constexpr (EXT == 2) return discriminant_fp64_proj_at<T>(in.C.R, pm, p0, pp, UXP);
-                    else if constexpr (EXT == 1) return discriminant_df_at<T>(in.C.R, in.C.well, pm, p0, pp, UXP, cind);
-                    else return discriminant_df_at<T>(CC.R, CC.well, pm, p0, pp, UXP, cind);
+                    else if constexpr (EXT == 1) return discriminant_df_at<T>(in.C.R, in.C.well, pm, p0, pp, 1, UXP, -UXP, cind);
+                    else return discriminant_df_at<T>(CC.R, CC.well, pm, p0, pp, 1, UXP, -UXP, cind);
                 };
                 if constexpr (MODE == MODE_ENERGY) {
-                    const T e = voxel_eval<T, false, EXT != 0, EXT == 2, SYM>(CC, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, ctv, refine);
+                    const T e = voxel_eval<T, false, EXT != 0, EXT == 2>(CC, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, ctv, refine);
                     if constexpr (kRow) se = fma_(wI, e, se);
                     return;
                 } else {
-                    const T e = voxel_eval<T, true, EXT != 0, EXT == 2, SYM, SYM>(CC, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, ctv, refine);
+                    const T e = voxel_eval<T, true, EXT != 0, EXT == 2>(CC, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, ctv, refine);
                     if constexpr (kOwn && kRow) se = fma_(wI, e, se);
                     // transposed-stencil pieces of this voxel (see the gather):
                     //   x/y first+second differences read from the left/right neighbour,
                     //   z pieces from the planes below/above, the centre term stays here
-                    //   (SYM: ctv.dx, dy, dz come without the stencil scale sg, which
-                    //   the FMAs below apply: 2 % faster there, 1 % slower in the
-                    //   general sweep, which keeps the scaled form)
-                    T X1, X2, Y1, Y2, zd, zu;
-                    if constexpr (SYM) {
-                        const T sgv = CC.sg;
-                        X1 = fma_(sgv, ctv.dx, ctv.hxx); X2 = fma_(-sgv, ctv.dx, ctv.hxx);
-                        Y1 = fma_(sgv, ctv.dy, ctv.hyy); Y2 = fma_(-sgv, ctv.dy, ctv.hyy);
-                        zd = fma_(sgv, ctv.dz, ctv.hzz); zu = fma_(-sgv, ctv.dz, ctv.hzz);
-                    } else {
-                        X1 = ctv.dx + ctv.hxx; X2 = ctv.hxx - ctv.dx;
-                        Y1 = ctv.dy + ctv.hyy; Y2 = ctv.hyy - ctv.dy;
-                        zd = ctv.dz + ctv.hzz; zu = ctv.hzz - ctv.dz;
-                    }
+                    const T X1 = ctv.dx + ctv.hxx, X2 = ctv.hxx - ctv.dx;
+                    const T Y1 = ctv.dy + ctv.hyy, Y2 = ctv.hyy - ctv.dy;
+                    const T zd = ctv.dz + ctv.hzz, zu = ctv.hzz - ctv.dz;
                     const T cpart = ctv.u - T(2) * (ctv.hxx + ctv.hyy + ctv.hzz);
                     if constexpr (kPublish) {   // plane m-1 is complete
                         cpend = accC + zu;
@@ -449,36 +393,34 @@ k_fused(const __grid_constant__ Launch<T, MAXI> L)
         };
         if (warp < TY) body(Y{}); else body(N{});
     }
-    if (cur >= 0) flush();
+    const T v[NPART] = { se, su, sg, sag, gmax, sout };
+    block_sums<NT>(v, scr, tot);
+    finish_problem(in, (int)blockIdx.x - in.first_block, MODE, tot);
 }
 
 size_t fused_smem_bytes(int elem_size, int tile_y);
 
 // One launch of k_fused (sets the dynamic shared-memory limit once per
 // instantiation; idempotent, so a race between threads is harmless).
-template <typename T, int TY, int MODE, int MAXI, int EXT = 0, bool SYM = false, bool HALO = false, bool UNI = false>
-static cudaError_t launch_kernel(const Launch<T, MAXI>& L, int blocks, cudaStream_t s)
+template <typename T, int TY, int MODE, int EXT = 0, bool HALO = false>
+static cudaError_t launch_kernel(const Launch<T, 1>& L, int blocks, cudaStream_t s)
 {
     const size_t smem = fused_smem_bytes(sizeof(T), TY);
     static bool attr_done = false;
     if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k_fused<T, TY, MODE, MAXI, EXT, SYM, HALO, UNI>,
+        cudaError_t e = cudaFuncSetAttribute(k_fused<T, TY, MODE, EXT, HALO>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    k_fused<T, TY, MODE, MAXI, EXT, SYM, HALO, UNI><<<blocks, Tile<TY>::NT, smem, s>>>(L);
+    k_fused<T, TY, MODE, EXT, HALO><<<blocks, Tile<TY>::NT, smem, s>>>(L);
     return cudaGetLastError();
 }
 
-// Batched launches whose problems share L.C0 and L.tau0 (pfc_fused_uni.cu);
-// sym: the SYM instantiation.
-cudaError_t launch_fused_uni(const Launch<float, BATCH_MAX>& L, int tile_y, int mode, bool sym, cudaStream_t s);
-
 // Split the launch's work units evenly over G CTAs and record, per problem,
 // the first CTA that holds a partial of it and how many do.
-template <typename T, int MAXI>
-static void plan(Launch<T, MAXI>& L, int tile_y, int max_run)
+template <typename T>
+static void plan(Launch<T, 1>& L, int tile_y, int max_run)
 {
     long long W = 0;
     for (int k = 0; k < L.n; ++k) {
@@ -504,9 +446,5 @@ static void plan(Launch<T, MAXI>& L, int tile_y, int max_run)
 // general instantiation (pfc_fused_slab.cu).
 template <typename T>
 cudaError_t launch_fused_halo(const Inst<T>& in, int mode, int tile_y, int max_run, cudaStream_t s);
-
-// The FP32 sweep for launches whose problems all have c3 = c5 = 0 (pfc_fused_sym.cu).
-template <int MAXI>
-cudaError_t launch_fused_sym(const Launch<float, MAXI>& L, int tile_y, int mode, cudaStream_t s);
 
 }  // namespace pfc

@@ -14,9 +14,9 @@ static cudaError_t launch_halo_mode(const Inst<T>& in, int mode, int max_run, cu
     L.inst[0] = in;
     plan(L, TY, max_run);
     switch (mode) {
-    case MODE_ENERGY: return launch_kernel<T, TY, MODE_ENERGY, 1, EXT, false, true>(L, L.grid, s);
-    case MODE_GRAD: return launch_kernel<T, TY, MODE_GRAD, 1, EXT, false, true>(L, L.grid, s);
-    case MODE_STEP: return launch_kernel<T, TY, MODE_STEP, 1, EXT, false, true>(L, L.grid, s);
+    case MODE_ENERGY: return launch_kernel<T, TY, MODE_ENERGY, EXT, true>(L, L.grid, s);
+    case MODE_GRAD: return launch_kernel<T, TY, MODE_GRAD, EXT, true>(L, L.grid, s);
+    case MODE_STEP: return launch_kernel<T, TY, MODE_STEP, EXT, true>(L, L.grid, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -27,9 +27,16 @@ cudaError_t launch_fused_halo(const Inst<T>& in, int mode, int tile_y, int max_r
     if (in.cf) return cudaErrorInvalidValue;   // slabs carry no coefficient field
     if (in.C.proj) return launch_halo_mode<T, EXT_TILE_Y, 2>(in, mode, max_run, s);
     if (needs_ext(in)) return launch_halo_mode<T, EXT_TILE_Y, 1>(in, mode, max_run, s);
-    if (tile_y == 8) return launch_halo_mode<T, 8, 0>(in, mode, max_run, s);
-    if (tile_y == 13) return launch_halo_mode<T, 13, 0>(in, mode, max_run, s);
-    return launch_halo_mode<T, 16, 0>(in, mode, max_run, s);
+    if constexpr (std::is_same<T, float>::value) {
+        Launch<float, 1> L;
+        L.n = 1;
+        L.inst[0] = in;
+        return launch_pair_halo(L, mode, tile_y, max_run, s);
+    } else {
+        if (tile_y == 8) return launch_halo_mode<T, 8, 0>(in, mode, max_run, s);
+        if (tile_y == 13) return launch_halo_mode<T, 13, 0>(in, mode, max_run, s);
+        return launch_halo_mode<T, 16, 0>(in, mode, max_run, s);
+    }
 }
 template cudaError_t launch_fused_halo<float>(const Inst<float>&, int, int, int, cudaStream_t);
 template cudaError_t launch_fused_halo<double>(const Inst<double>&, int, int, int, cudaStream_t);

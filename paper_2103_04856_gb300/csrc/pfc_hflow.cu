@@ -978,7 +978,7 @@ extern "C" pfc_status pfc_hflow_create(const pfc_problem* prob, const pfc_hflow_
         }
     }
     cudaGetDevice(&h->device);
-    h->sweep_slots = (int)fused_slots(p.nx, p.ny, p.nz, h->tile_y, p.tile_z);
+    h->sweep_slots = (int)fused_grid(fused_units(p.nx, p.ny, p.nz), p.tile_z);
     bool ok = true;
     for (void*& b : h->buf) ok = ok && cudaMalloc(&b, (size_t)h->esz * h->N) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&h->spart, sizeof(double) * NPART * (size_t)h->sweep_slots) == cudaSuccess &&
@@ -1454,8 +1454,7 @@ extern "C" pfc_status pfc_hflow_batch_create(const pfc_problem* probs, const dou
     }
     b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(b->ny, false);
     cudaGetDevice(&b->device);
-    const long long units = (long long)((b->nx + 31) / 32) * ((b->ny + b->tile_y - 1) / b->tile_y) * b->nz * n_inst;
-    b->slots = (int)fused_grid(units, probs[0].tile_z);
+    b->slots = (int)fused_grid(fused_units(b->nx, b->ny, b->nz) * n_inst, probs[0].tile_z);
     b->fblocks = flow_blocks(b->N);
     const size_t n = (size_t)n_inst;
     bool ok = cudaMalloc((void**)&b->bufs, sizeof(float) * 4 * (size_t)b->N * n) == cudaSuccess &&

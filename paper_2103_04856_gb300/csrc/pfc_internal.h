@@ -56,6 +56,14 @@ struct Coef {
     // where 2S + T^2 > rthr max(|D|, xi) and D is finite (voxel_eval):
     // rthr = 2^16, or infinity to never refine
     T rthr;
+    // The packed FP32 sweep's constants for symmetric polynomials, on raw
+    // differences (pair_eval_sym), from FP64 products.  K = 1 / (eps kd); wells
+    // 0/1: wA = -12 K, wB = 2 K; wells -1/1: wA = 3 K, wB = -K
+    T wA, wB;
+    // c1 kd^2, c2 kd^2, c4 sg kd / 2, c6 sg^2, xi^2 / sg^2; nform: sym, and all
+    // of them are representable (else the general form runs)
+    T n1, n2, n4, n6, nx2;
+    int nform;
 };
 
 // Coefficient fields: c(x) = (c1..c6)(a(x)) as 6 component planes of N
@@ -74,6 +82,10 @@ struct Inst {
     int first_block;     // plain path: unused; fused: first CTA holding a partial of this problem
     int nblocks;         // number of FP64 partial slots (CTAs) of this problem in the launch
     long long unit_base; // fused: first work unit (one plane of one column tile) of this problem
+    // fused: the weight of the units before it, and of a unit of its first
+    // tiles_full tiles and of the others (the ragged last row of tiles)
+    long long wbase;
+    int tiles_full, w_full, w_last;
     Coef<T> C;
     const T* cf;         // null, or the coefficient field c(x) [NCF][nz][ny][nx] replacing C.c1..c6
     T tau;
@@ -96,18 +108,15 @@ struct Inst {
 // descriptors are read from the constant bank, uniformly per CTA).
 constexpr int BATCH_MAX = 64;
 // Work is split in units of one z-plane of one 32 x TY column tile,
-// enumerated problem by problem, tile by tile, plane by plane; CTA b of G
-// takes units [b W / G, (b+1) W / G).
+// enumerated problem by problem, tile by tile, plane by plane, each with a
+// weight (1, or what its warps cost where a ragged tile leaves some idle);
+// CTA b of G takes the units that start in [b W / G, (b+1) W / G) of the
+// total weight W.
 template <typename T, int MAXI>
 struct Launch {
     int n;
     int grid;            // G
-    long long units;     // W
-    // launches whose problems share one coefficient set and step size
-    // (k_fused<..., UNI = true>) read them here, at a fixed offset of the
-    // constant bank, instead of from inst[k] at a run-time index
-    Coef<T> C0;
-    T tau0;
+    long long units;     // W, the weights of all units
     Inst<T> inst[MAXI];
 };
 
@@ -115,19 +124,15 @@ template <typename T>
 Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, double mu = 0.0,
                   const double* theta = nullptr, int proj = 0, int refine = 1);
 
-// Automatic tile height: FP64 8 rows; FP32 the one of 16 and 13 rows that
-// pads the grid's rows least (16 on a tie: its tiles hold more rows), except
-// for general polynomials (not symmetric in kappa1, kappa2), whose 16-row
-// instantiation keeps more values in local memory than the 13-row one: a row
-// of it costs 4 % more (a 256^3 problem, pfc_run: 0.2354 ms per step at 16
-// rows, 0.2295 ms at 13 with 260 rows), so they take 13 rows unless 16 pads
-// more than 4 % less.
-inline int default_tile_y(int ny, bool fp64, bool general = false)
+// Tile rows of the packed FP32 sweep (k_pair) for a height hint
+// (pfc_problem.tile_y): its tiles hold an even number of rows.
+inline int pair_tile_rows(int tile_y) { return tile_y == 8 ? 8 : tile_y == 13 ? 12 : 20; }
+
+// Automatic tile height (as a hint): FP64 8 rows, FP32 the tallest.
+inline int default_tile_y(int ny, bool fp64)
 {
-    if (fp64) return 8;
-    const int pad16 = (ny + 15) / 16 * 16, pad13 = (ny + 12) / 13 * 13;
-    if (general) return pad13 < 1.04 * pad16 ? 13 : 16;
-    return pad13 < pad16 ? 13 : 16;
+    (void)ny;
+    return fp64 ? 8 : 16;
 }
 
 // The extended sweep (orientation term, c(x), projected M) runs with 8-row tiles.
@@ -153,9 +158,17 @@ cudaError_t launch_fused(const Inst<T>& in, int mode, int tile_y, int max_run, c
 cudaError_t launch_fused_batch(const Inst<float>* insts, int n_inst, int tile_y, int max_run, cudaStream_t s,
                                int mode = MODE_STEP);
 long long fused_grid(long long units, int max_run);
-// partial slots a single problem can need: both the requested tile height and
-// the extended sweep's
-long long fused_slots(int nx, int ny, int nz, int tile_y, int max_run);
+// Work units of a problem in tiles of 8 rows, the shortest of any sweep: a
+// launch of it never has more CTAs, hence partial slots, than
+// fused_grid(fused_units(...), max_run).
+long long fused_units(int nx, int ny, int nz);
+// the packed FP32 sweep (pfc_pair*.cu): plans the launch's tiles for the
+// height hint tile_y and runs it; general and symmetric polynomials, z-slabs
+template <int MAXI>
+cudaError_t launch_pair(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s);
+template <int MAXI>
+cudaError_t launch_pair_sym(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s);
+cudaError_t launch_pair_halo(Launch<float, 1>& L, int mode, int tile_y, int max_run, cudaStream_t s);
 template <typename T>
 cudaError_t launch_add_offset(T* out, const T* in, long n, const double* c, cudaStream_t s);
 // out += scal[S_C] for every problem of a batch (host descriptors), in place

@@ -118,7 +118,7 @@ static pfc_status run_noalloc(const pfc_problem* p, const void* u, void* g, doub
     in.ints = (unsigned*)(base + kPartBytes + kScalBytes);
     in.trace = nullptr;
     in.trace_cap = 0;
-    if (fused_slots(p->nx, p->ny, p->nz, tile_y, p->tile_z) > kMaxCtas)
+    if (fused_grid(fused_units(p->nx, p->ny, p->nz), p->tile_z) > kMaxCtas)
         return na_fail(PFC_EINVAL, "noalloc: the launch would need more than 1024 CTAs of scratch "
                                    "(lower tile_z or use pfc_energy_and_grad)");
     // the counters must start at zero; everything else is written before it is read

@@ -1,0 +1,260 @@
+// pfc_pair.cuh -- two voxels at a time: packed FP32 arithmetic (one
+// instruction on two floats in a 64-bit register) and eq. Feps with its local
+// reverse mode on a pair of voxels.
+//
+// The FP32 sweep is bound by instruction issue, not by the FP32 pipe: a third
+// of its instructions are loads, stores, addresses and barriers.  A packed
+// multiply-add occupies the pipe for as long as two scalar ones (measured: the
+// same FLOP rate) but takes one issue slot, and the loads and addresses of a
+// pair are shared, so the same voxels need about half the slots.
+#pragma once
+
+#include "pfc_device.cuh"
+
+namespace pfc {
+
+struct __align__(8) F2 {
+    unsigned long long b;    // low word: the first voxel
+};
+
+__device__ __forceinline__ F2 pk(float lo, float hi)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.b) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ F2 dup(float x) { return pk(x, x); }
+__device__ __forceinline__ float lo(F2 a)
+{
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.b));
+    return x;
+}
+__device__ __forceinline__ float hi(F2 a)
+{
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.b));
+    return y;
+}
+__device__ __forceinline__ F2 operator+(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(a.b), "l"(b.b));
+    return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b)
+{
+    F2 r;
+    asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(a.b), "l"(b.b));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(a.b), "l"(b.b));
+    return r;
+}
+__device__ __forceinline__ F2 fma_(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.b) : "l"(a.b), "l"(b.b), "l"(c.b));
+    return r;
+}
+
+// Half the cotangents of a pair of voxels with respect to the raw stencil
+// values (see Cot); the mixed ones without their factor 1/2 (each feeds M_cd
+// and M_dc with the four-point difference's 1/4).
+struct Cot2 {
+    F2 u, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz;
+};
+
+// Coefficients of eq. Feps and the stencil scales as pairs, for the general
+// form, formed once per run.
+struct Coef2 {
+    F2 c1, c2, c3, c4, c5, c6, c1x2, c2x2, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
+    float xi, xi64, inv_xi, rthr;
+    int well;
+};
+__device__ __forceinline__ Coef2 coef2(const Coef<float>& C)
+{
+    Coef2 P;
+    P.c1 = dup(C.c1); P.c2 = dup(C.c2); P.c3 = dup(C.c3); P.c4 = dup(C.c4); P.c5 = dup(C.c5); P.c6 = dup(C.c6);
+    P.c1x2 = dup(C.c1x2); P.c2x2 = dup(C.c2x2); P.c6x2 = dup(C.c6x2);
+    P.kd = dup(C.kd); P.ko = dup(C.ko); P.ko2 = dup(C.ko2); P.sg = dup(C.sg); P.nsg = dup(-C.sg);
+    P.ie = dup(C.inv_eps); P.xi2 = dup(C.xi2);
+    P.xi = C.xi; P.xi64 = 64.0f * C.xi; P.inv_xi = C.inv_xi; P.rthr = C.rthr;
+    P.well = C.well;
+    return P;
+}
+
+__device__ __forceinline__ float ex2_(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// log(1 + x) for x in [0, 1]: x times a degree-9 minimax fit of log(1 + x) / x
+// (reweighted least squares in Chebyshev polynomials on [0, 1], relative error
+// 4.7e-9; with FP32 rounding at most 1.5e-7).
+__device__ __forceinline__ F2 log1p01(F2 x)
+{
+    F2 p = fma_(dup(-3.244023304e-03f), x, dup(1.985145360e-02f));
+    p = fma_(p, x, dup(-5.695951730e-02f));
+    p = fma_(p, x, dup(1.060365364e-01f));
+    p = fma_(p, x, dup(-1.530559212e-01f));
+    p = fma_(p, x, dup(1.967593879e-01f));
+    p = fma_(p, x, dup(-2.495413423e-01f));
+    p = fma_(p, x, dup(3.332996368e-01f));
+    p = fma_(p, x, dup(-4.999990165e-01f));
+    p = fma_(p, x, dup(1.0f));
+    return p * x;
+}
+
+// sqrt(P(D)) and d sqrt(P) / dD of both voxels (softplus_, one reciprocal
+// square root for both; 0 where P underflows to 0), without branches: where
+// softplus_ drops the correction (|D| > 64 xi) ex is set to 0.
+__device__ __forceinline__ void root_softplus(float D0, float D1, const Coef2& C, F2& r, F2& rp)
+{
+    const float a0 = fabsf(D0), a1 = fabsf(D1);
+    const F2 t = pk(a0, a1) * dup(-C.inv_xi) * dup(1.4426950408889634f);
+    float e0 = ex2_(lo(t)), e1 = ex2_(hi(t));
+    e0 = a0 > C.xi64 ? 0.0f : e0;
+    e1 = a1 > C.xi64 ? 0.0f : e1;
+    const F2 ex = pk(e0, e1), den = ex + dup(1.0f);
+    const F2 inv = pk(__fdividef(1.0f, lo(den)), __fdividef(1.0f, hi(den)));
+    const F2 exi = ex * inv;
+    const F2 P = fma_(dup(C.xi), log1p01(ex), pk(fmaxf(D0, 0.0f), fmaxf(D1, 0.0f)));
+    const F2 Pp = pk(D0 >= 0.0f ? lo(inv) : lo(exi), D1 >= 0.0f ? hi(inv) : hi(exi));
+    const F2 rs = pk(rsqrtf(fmaxf(lo(P), 1e-37f)), rsqrtf(fmaxf(hi(P), 1e-37f)));
+    r = P * rs;
+    rp = dup(0.5f) * Pp * rs;
+}
+
+// voxel_eval's eq. Meps path on a pair: the same operations in the same order
+// and rounding (D's last bits decide sqrt(D+) at the kink); ct.dx, dy, dz come
+// without the stencil scale sg.
+// refine(h): D of the pair's voxel h (0 or 1) in double-float.
+template <bool GRAD, class Refine>
+__device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 dz, F2 hxx, F2 hyy, F2 hzz, F2 hxy,
+                                        F2 hxz, F2 hyz, Cot2& ct, const Refine& refine)
+{
+    const F2 one = dup(1.0f), two = dup(2.0f), mone = dup(-1.0f), mtwo = dup(-2.0f);
+    const F2 Gx = dx * C.sg, Gy = dy * C.sg, Gz = dz * C.sg;
+    const F2 g2 = fma_(Gx, Gx, fma_(Gy, Gy, Gz * Gz));
+    const F2 rho = g2 + C.xi2;
+    const F2 iq = pk(rsqrtf(lo(rho)), rsqrtf(hi(rho)));
+    const F2 q = rho * iq;
+    const F2 irho = iq * iq;
+    F2 wp, wpp;              // W'(u), W''(u)
+    if (C.well == 0) {
+        const F2 t = fma_(u0 * mone, u0, u0);                 // u (1 - u)
+        wp = (t * two) * fma_(u0, mtwo, one);
+        wpp = fma_(t, dup(-12.0f), two);                      // 2 (1 - 6u + 6u^2)
+    } else {
+        const F2 uu = u0 * u0;
+        wp = fma_(uu, u0, u0 * mone);
+        wpp = fma_(dup(3.0f) * u0, u0, mone);
+    }
+    const F2 wr = wp * C.ie * irho;                           // (W'/eps) / rho
+    const F2 wx = wr * Gx, wy = wr * Gy, wz = wr * Gz;
+    const F2 Mxx = fma_(C.kd, hxx, wx * Gx), Myy = fma_(C.kd, hyy, wy * Gy), Mzz = fma_(C.kd, hzz, wz * Gz);
+    const F2 Mxy = fma_(C.ko, hxy, wx * Gy), Mxz = fma_(C.ko, hxz, wx * Gz), Myz = fma_(C.ko, hyz, wy * Gz);
+    const F2 Tr = Mxx + Myy + Mzz;
+    const F2 off = fma_(Mxy, Mxy, fma_(Mxz, Mxz, Myz * Myz));
+    const F2 S = fma_(Mxx, Mxx, fma_(Myy, Myy, fma_(Mzz, Mzz, off + off)));
+    const F2 t2 = Tr * Tr;
+    const F2 c4q = C.c4 * q;
+    const F2 a3 = fma_(C.c3, Tr, C.c5 * q);
+    const F2 nt2 = t2 * mone;
+    const F2 t2e = fma_(Tr, Tr, nt2);                         // the rounding error of T^2, put back
+    const F2 D = fma_(two, S, nt2) - t2e;
+    const F2 scale = fma_(two, S, t2);
+    float D0 = lo(D), D1 = hi(D);
+    const bool n0 = lo(a3) != 0.0f && lo(scale) > C.rthr * fmax_nan_(fabsf(D0), C.xi);
+    const bool n1 = hi(a3) != 0.0f && hi(scale) > C.rthr * fmax_nan_(fabsf(D1), C.xi);
+    if (n0 || n1) {
+        if (n0) D0 = refine(0);
+        if (n1) D1 = refine(1);
+    }
+    F2 r, rp;
+    root_softplus(D0, D1, C, r, rp);
+    const F2 e = fma_(C.c1, S, fma_(C.c2, t2, fma_(a3, r, fma_(c4q, Tr, C.c6 * g2))));
+    if constexpr (!GRAD) return e;
+    const F2 k = a3 * rp;                                     // de/dD
+    const F2 dT = fma_(C.c2x2, Tr, fma_(C.c3, r, fma_(C.c4, q, (Tr * mtwo) * k)));
+    const F2 dq = fma_(C.c4, Tr, C.c5 * r);
+    const F2 s2 = two * fma_(two, k, C.c1);
+    // Lambda = de/dM = 2 dS M + dT I
+    const F2 Lxx = fma_(s2, Mxx, dT), Lyy = fma_(s2, Myy, dT), Lzz = fma_(s2, Mzz, dT);
+    const F2 Lxy = s2 * Mxy, Lxz = s2 * Mxz, Lyz = s2 * Myz;
+    const F2 LGx = fma_(Lxx, Gx, fma_(Lxy, Gy, Lxz * Gz));
+    const F2 LGy = fma_(Lxy, Gx, fma_(Lyy, Gy, Lyz * Gz));
+    const F2 LGz = fma_(Lxz, Gx, fma_(Lyz, Gy, Lzz * Gz));
+    const F2 GLG = fma_(Gx, LGx, fma_(Gy, LGy, Gz * LGz));
+    ct.u = wpp * C.ie * GLG * irho;
+    const F2 al = wr * two;
+    const F2 be = fma_((wr * mtwo) * GLG, irho, fma_(dq, iq, C.c6x2));
+    ct.dx = fma_(al, LGx, be * Gx);
+    ct.dy = fma_(al, LGy, be * Gy);
+    ct.dz = fma_(al, LGz, be * Gz);
+    ct.hxx = C.kd * Lxx; ct.hyy = C.kd * Lyy; ct.hzz = C.kd * Lzz;
+    ct.hxy = C.ko2 * Lxy; ct.hxz = C.ko2 * Lxz; ct.hyz = C.ko2 * Lyz;   // Hess_cd feeds M_cd and M_dc
+    return e;
+}
+
+// The density and half its cotangents (Cot2) for c3 = c5 = 0, on the raw differences d = grad u / sg: with
+// M = kd N and G = sg d, N_cc = h_cc + w d_c d_c and N_cd = h_cd / 4 + w d_c
+// d_d, w = W' / (eps kd) / (|d|^2 + xi^2 / sg^2); e = n1 ||N||^2 + n2 T^2 +
+// 2 n4 q T + n6 |d|^2 with q = sqrt(|d|^2 + xi^2 / sg^2).  No stencil scale is
+// applied and no second difference multiplied: 14 products fewer.
+template <bool GRAD>
+__device__ __forceinline__ F2 pair_eval_sym(const Coef<float>& C, F2 u0, F2 dx, F2 dy, F2 dz, F2 hxx, F2 hyy, F2 hzz,
+                                            F2 hxy, F2 hxz, F2 hyz, Cot2& ct)
+{
+    const F2 one = dup(1.0f), quarter = dup(0.25f), n1 = dup(C.n1);
+    const F2 g2 = fma_(dx, dx, fma_(dy, dy, dz * dz));
+    const F2 rho = g2 + dup(C.nx2);
+    const F2 iq = pk(rsqrtf(lo(rho)), rsqrtf(hi(rho)));
+    const F2 q = rho * iq;
+    const F2 irho = iq * iq;
+    F2 wp, wpk;              // W'(u) / wB K, W''(u) K
+    if (C.well == 0) {
+        const F2 v = one - u0;
+        const F2 t = u0 * v;                                  // W' = 2 t (1 - 2u), W'' = 2 - 12 t
+        wp = t * (v - u0);
+        wpk = fma_(t, dup(C.wA), dup(C.wB));
+    } else {
+        const F2 uu = u0 * u0;                                // W' = -u (1 - u^2), W'' = 3 u^2 - 1
+        wp = u0 * (one - uu);
+        wpk = fma_(uu, dup(C.wA), dup(C.wB));
+    }
+    const F2 w = wp * dup(C.wB) * irho;
+    const F2 wx = w * dx, wy = w * dy, wz = w * dz;
+    const F2 Nxx = fma_(wx, dx, hxx), Nyy = fma_(wy, dy, hyy), Nzz = fma_(wz, dz, hzz);
+    const F2 Nxy = fma_(quarter, hxy, wx * dy), Nxz = fma_(quarter, hxz, wx * dz), Nyz = fma_(quarter, hyz, wy * dz);
+    const F2 Tr = Nxx + Nyy + Nzz;
+    const F2 off = fma_(Nxy, Nxy, fma_(Nxz, Nxz, Nyz * Nyz));
+    const F2 S = fma_(Nxx, Nxx, fma_(Nyy, Nyy, fma_(Nzz, Nzz, off + off)));
+    const F2 q4 = dup(C.n4) * q;
+    const F2 dT = fma_(dup(C.n2), Tr, q4);                    // half of de/dT
+    const F2 e = fma_(n1, S, fma_(Tr, dT + q4, dup(C.n6) * g2));
+    if constexpr (!GRAD) return e;
+    const F2 Lxx = fma_(n1, Nxx, dT), Lyy = fma_(n1, Nyy, dT), Lzz = fma_(n1, Nzz, dT);
+    const F2 Lxy = n1 * Nxy, Lxz = n1 * Nxz, Lyz = n1 * Nyz;
+    const F2 LGx = fma_(Lxx, dx, fma_(Lxy, dy, Lxz * dz));
+    const F2 LGy = fma_(Lxy, dx, fma_(Lyy, dy, Lyz * dz));
+    const F2 LGz = fma_(Lxz, dx, fma_(Lyz, dy, Lzz * dz));
+    const F2 GLG = fma_(dx, LGx, fma_(dy, LGy, dz * LGz));
+    ct.u = wpk * GLG * irho;
+    const F2 al = w + w;
+    const F2 be = fma_(dup(C.n4) * Tr, iq, dup(C.n6)) - al * GLG * irho;
+    ct.dx = fma_(al, LGx, be * dx);
+    ct.dy = fma_(al, LGy, be * dy);
+    ct.dz = fma_(al, LGz, be * dz);
+    ct.hxx = Lxx; ct.hyy = Lyy; ct.hzz = Lzz;
+    ct.hxy = Lxy; ct.hxz = Lxz; ct.hyz = Lyz;
+    return e;
+}
+
+}  // namespace pfc
