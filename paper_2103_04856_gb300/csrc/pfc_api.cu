@@ -70,9 +70,11 @@ struct pfc_ctx {
     double* dpart = nullptr;         // diagnostics: block partials, ticket, 5 results
     unsigned* dticket = nullptr;
     double* dout = nullptr;
-    void* skap = nullptr;            // surface cells: kappa1, kappa2 fields, block counts, offsets
+    void* skap = nullptr;            // surface cells: kappa1, kappa2 fields, counts and masks, offsets
     unsigned* sblk = nullptr;
     long long* soff = nullptr;
+    double* hpart = nullptr;         // curvature histogram: hcap doubles of partial tables
+    size_t hcap = 0;
     // cached step-loop graph
     cudaGraphExec_t gexec = nullptr;
     const void* g_u = nullptr;
@@ -181,6 +183,7 @@ static void free_ctx_mem(pfc_ctx* c)
     cudaFree(c->skap);
     cudaFree(c->sblk);
     cudaFree(c->soff);
+    cudaFree(c->hpart);
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->cap) cudaStreamDestroy(c->cap);
 }
@@ -564,14 +567,17 @@ extern "C" pfc_status pfc_surface_cells(pfc_ctx* c, const void* u, double level,
     if (st) return st;
     if (cap > 0 && (st = check_dev_ptr(c, cells, "cells"))) return st;
     const long nb = surface_blocks(c->N);
-    if (!c->skap) {
-        PFC_CU(cudaMalloc(&c->skap, (size_t)c->esz * 2 * c->N));
-        PFC_CU(cudaMalloc((void**)&c->sblk, sizeof(unsigned) * (size_t)nb));
-        PFC_CU(cudaMalloc((void**)&c->soff, sizeof(long long) * (size_t)(nb + 1)));
-    }
+    if (!c->soff) PFC_CU(cudaMalloc((void**)&c->soff, sizeof(long long) * (size_t)(nb + 1)));
+    if (cap > 0 && !c->sblk) PFC_CU(cudaMalloc((void**)&c->sblk, sizeof(unsigned) * (size_t)surface_work(c->N)));
+    if (cap > 0 && !c->skap) PFC_CU(cudaMalloc(&c->skap, (size_t)c->esz * 2 * c->N));
     cudaStream_t s = (cudaStream_t)stream;
     const pfc_problem& P = c->P;
-    if (P.prec == PFC_FP64) {
+    if (cap == 0) {   // the number of cells only
+        if (P.prec == PFC_FP64)
+            PFC_CU(launch_surface_count<double>((const double*)u, P.nx, P.ny, P.nz, level, c->soff + nb, s));
+        else
+            PFC_CU(launch_surface_count<float>((const float*)u, P.nx, P.ny, P.nz, level, c->soff + nb, s));
+    } else if (P.prec == PFC_FP64) {
         double* k1 = (double*)c->skap;
         double* k2 = k1 + c->N;
         PFC_CU(launch_curvatures<double>((const double*)u, k1, k2, P.nx, P.ny, P.nz,
@@ -603,10 +609,21 @@ extern "C" pfc_status pfc_curvature_histogram(pfc_ctx* c, const void* cells, int
     if (st) return st;
     if (n > 0 && (st = check_dev_ptr(c, cells, "cells"))) return st;
     cudaStream_t s = (cudaStream_t)stream;
+    const int copies = histogram_copies(nbins);
+    const size_t need = copies > 1 ? (size_t)copies * nbins * nbins : 0;
+    if (need > c->hcap) {   // grown only: at most 16 MB
+        PFC_CU(cudaStreamSynchronize(s));
+        cudaFree(c->hpart);
+        c->hpart = nullptr;
+        c->hcap = 0;
+        PFC_CU(cudaMalloc((void**)&c->hpart, sizeof(double) * need));
+        c->hcap = need;
+    }
+    double* part = need ? c->hpart : nullptr;
     if (c->P.prec == PFC_FP64)
-        PFC_CU(launch_curvature_histogram<double>((const double*)cells, n, nbins, lo, hi, hist_dev, s));
+        PFC_CU(launch_curvature_histogram<double>((const double*)cells, n, nbins, lo, hi, part, hist_dev, s));
     else
-        PFC_CU(launch_curvature_histogram<float>((const float*)cells, n, nbins, lo, hi, hist_dev, s));
+        PFC_CU(launch_curvature_histogram<float>((const float*)cells, n, nbins, lo, hi, part, hist_dev, s));
     return PFC_OK;
 }
 

@@ -192,16 +192,23 @@ template <typename T>
 cudaError_t launch_diagnostics(const T* u, int nx, int ny, int nz, double h, double eps, int well, double* part,
                                unsigned* ticket, double* out, cudaStream_t s);
 
-// curvature-diagram cells (pfc_surface.cu): block_counts holds
-// surface_blocks(n) values, offsets surface_blocks(n) + 1 (the total last);
-// cells receive min(total, cap) records (area, kappa1, kappa2)
+// curvature-diagram cells (pfc_surface.cu): work holds surface_work(n) values
+// (counts and corner masks), offsets surface_blocks(n) + 1 (the total last);
+// cells receive min(total, cap) records (area, kappa1, kappa2).
+// launch_surface_count: their number alone, into *total (device)
 long surface_blocks(long n);
+long surface_work(long n);
+template <typename T>
+cudaError_t launch_surface_count(const T* u, int nx, int ny, int nz, double level, long long* total, cudaStream_t s);
 template <typename T>
 cudaError_t launch_surface_cells(const T* u, const T* k1, const T* k2, int nx, int ny, int nz, double h, double level,
-                                 unsigned* block_counts, long long* offsets, T* cells, long long cap, cudaStream_t s);
+                                 unsigned* work, long long* offsets, T* cells, long long cap, cudaStream_t s);
+// part: histogram_copies(nbins) tables of nbins^2 values to work in, or null
+// where that is 1
+int histogram_copies(int nbins);
 template <typename T>
-cudaError_t launch_curvature_histogram(const T* cells, long long n, int nbins, double lo, double hi, double* hist,
-                                       cudaStream_t s);
+cudaError_t launch_curvature_histogram(const T* cells, long long n, int nbins, double lo, double hi, double* part,
+                                       double* hist, cudaStream_t s);
 
 // plain unfused path (pfc_plain.cu)
 template <typename T>
