@@ -56,8 +56,8 @@ struct Coef {
     // where 2S + T^2 > rthr max(|D|, xi) and D is finite (voxel_eval):
     // rthr = 2^16, or infinity to never refine
     T rthr;
-    // The packed FP32 sweep's constants for symmetric polynomials, on raw
-    // differences (pair_eval_sym), from FP64 products.  K = 1 / (eps kd); wells
+    // Constants for symmetric polynomials on raw
+    // differences (eval_sym), from FP64 products.  K = 1 / (eps kd); wells
     // 0/1: wA = -12 K, wB = 2 K; wells -1/1: wA = 3 K, wB = -K
     T wA, wB;
     // c1 kd^2, c2 kd^2, c4 sg kd / 2, c6 sg^2, xi^2 / sg^2; nform: sym, and all
@@ -168,6 +168,7 @@ template <int MAXI>
 cudaError_t launch_pair(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s);
 template <int MAXI>
 cudaError_t launch_pair_sym(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s);
+cudaError_t launch_pair_ext(Launch<float, 1>& L, int mode, int max_run, cudaStream_t s);
 cudaError_t launch_pair_halo(Launch<float, 1>& L, int mode, int tile_y, int max_run, cudaStream_t s);
 template <typename T>
 cudaError_t launch_add_offset(T* out, const T* in, long n, const double* c, cudaStream_t s);

@@ -61,17 +61,30 @@ __device__ __forceinline__ F2 fma_(F2 a, F2 b, F2 c)
     return r;
 }
 
-// Half the cotangents of a pair of voxels with respect to the raw stencil
-// values (see Cot); the mixed ones without their factor 1/2 (each feeds M_cd
-// and M_dc with the four-point difference's 1/4).
-struct Cot2 {
-    F2 u, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz;
+// Half the cotangents with respect to the raw stencil values (see Cot) of a
+// pair of voxels (V = F2) or one FP64 voxel (V = double); the mixed ones
+// without their factor 1/2 (each feeds M_cd and M_dc with the four-point
+// difference's 1/4).
+template <class V>
+struct CotH {
+    V u, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz;
 };
+using Cot2 = CotH<F2>;
+
+// a number as a value of V; 1 / sqrt
+template <class V> __device__ __forceinline__ V bc(double x);
+template <> __device__ __forceinline__ F2 bc<F2>(double x) { return dup((float)x); }
+template <> __device__ __forceinline__ double bc<double>(double x) { return x; }
+__device__ __forceinline__ F2 bcv(F2, float x) { return dup(x); }
+__device__ __forceinline__ double bcv(double, double x) { return x; }
+__device__ __forceinline__ F2 rsq(F2 a) { return pk(rsqrtf(lo(a)), rsqrtf(hi(a))); }
+__device__ __forceinline__ double rsq(double a) { return rsqrt(a); }
 
 // Coefficients of eq. Feps and the stencil scales as pairs, for the general
 // form, formed once per run.
 struct Coef2 {
-    F2 c1, c2, c3, c4, c5, c6, c1x2, c2x2, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
+    F2 c1, c2, c3, c4, c5, c6, c2x2, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
+    F2 c7, c7x2, th0, th1, th2;       // orientation term (ORIENT)
     float xi, xi64, inv_xi, rthr;
     int well;
 };
@@ -79,7 +92,8 @@ __device__ __forceinline__ Coef2 coef2(const Coef<float>& C)
 {
     Coef2 P;
     P.c1 = dup(C.c1); P.c2 = dup(C.c2); P.c3 = dup(C.c3); P.c4 = dup(C.c4); P.c5 = dup(C.c5); P.c6 = dup(C.c6);
-    P.c1x2 = dup(C.c1x2); P.c2x2 = dup(C.c2x2); P.c6x2 = dup(C.c6x2);
+    P.c2x2 = dup(C.c2x2); P.c6x2 = dup(C.c6x2);
+    P.c7 = dup(C.c7); P.c7x2 = dup(2.0f * C.c7); P.th0 = dup(C.th0); P.th1 = dup(C.th1); P.th2 = dup(C.th2);
     P.kd = dup(C.kd); P.ko = dup(C.ko); P.ko2 = dup(C.ko2); P.sg = dup(C.sg); P.nsg = dup(-C.sg);
     P.ie = dup(C.inv_eps); P.xi2 = dup(C.xi2);
     P.xi = C.xi; P.xi64 = 64.0f * C.xi; P.inv_xi = C.inv_xi; P.rthr = C.rthr;
@@ -134,8 +148,9 @@ __device__ __forceinline__ void root_softplus(float D0, float D1, const Coef2& C
 // voxel_eval's eq. Meps path on a pair: the same operations in the same order
 // and rounding (D's last bits decide sqrt(D+) at the kink); ct.dx, dy, dz come
 // without the stencil scale sg.
+// ORIENT adds the orientation term of Sec. 5.2 (see voxel_eval).
 // refine(h): D of the pair's voxel h (0 or 1) in double-float.
-template <bool GRAD, class Refine>
+template <bool GRAD, bool ORIENT, class Refine>
 __device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 dz, F2 hxx, F2 hyy, F2 hzz, F2 hxy,
                                         F2 hxz, F2 hyz, Cot2& ct, const Refine& refine)
 {
@@ -179,7 +194,12 @@ __device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 
     }
     F2 r, rp;
     root_softplus(D0, D1, C, r, rp);
-    const F2 e = fma_(C.c1, S, fma_(C.c2, t2, fma_(a3, r, fma_(c4q, Tr, C.c6 * g2))));
+    F2 e = fma_(C.c1, S, fma_(C.c2, t2, fma_(a3, r, fma_(c4q, Tr, C.c6 * g2))));
+    F2 tg;
+    if constexpr (ORIENT) {
+        tg = fma_(C.th0, Gx, fma_(C.th1, Gy, C.th2 * Gz));
+        e = fma_(C.c7 * tg, tg, e);
+    }
     if constexpr (!GRAD) return e;
     const F2 k = a3 * rp;                                     // de/dD
     const F2 dT = fma_(C.c2x2, Tr, fma_(C.c3, r, fma_(C.c4, q, (Tr * mtwo) * k)));
@@ -198,6 +218,12 @@ __device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 
     ct.dx = fma_(al, LGx, be * Gx);
     ct.dy = fma_(al, LGy, be * Gy);
     ct.dz = fma_(al, LGz, be * Gz);
+    if constexpr (ORIENT) {
+        const F2 ot = C.c7x2 * tg;
+        ct.dx = fma_(ot, C.th0, ct.dx);
+        ct.dy = fma_(ot, C.th1, ct.dy);
+        ct.dz = fma_(ot, C.th2, ct.dz);
+    }
     ct.hxx = C.kd * Lxx; ct.hyy = C.kd * Lyy; ct.hzz = C.kd * Lzz;
     ct.hxy = C.ko2 * Lxy; ct.hxz = C.ko2 * Lxz; ct.hyz = C.ko2 * Lyz;   // Hess_cd feeds M_cd and M_dc
     return e;
@@ -208,47 +234,48 @@ __device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 
 // d_d, w = W' / (eps kd) / (|d|^2 + xi^2 / sg^2); e = n1 ||N||^2 + n2 T^2 +
 // 2 n4 q T + n6 |d|^2 with q = sqrt(|d|^2 + xi^2 / sg^2).  No stencil scale is
 // applied and no second difference multiplied: 14 products fewer.
-template <bool GRAD>
-__device__ __forceinline__ F2 pair_eval_sym(const Coef<float>& C, F2 u0, F2 dx, F2 dy, F2 dz, F2 hxx, F2 hyy, F2 hzz,
-                                            F2 hxy, F2 hxz, F2 hyz, Cot2& ct)
+template <bool GRAD, class V, class T>
+__device__ __forceinline__ V eval_sym(const Coef<T>& C, V u0, V dx, V dy, V dz, V hxx, V hyy, V hzz, V hxy, V hxz,
+                                      V hyz, CotH<V>& ct)
 {
-    const F2 one = dup(1.0f), quarter = dup(0.25f), n1 = dup(C.n1);
-    const F2 g2 = fma_(dx, dx, fma_(dy, dy, dz * dz));
-    const F2 rho = g2 + dup(C.nx2);
-    const F2 iq = pk(rsqrtf(lo(rho)), rsqrtf(hi(rho)));
-    const F2 q = rho * iq;
-    const F2 irho = iq * iq;
-    F2 wp, wpk;              // W'(u) / wB K, W''(u) K
+    auto k = [&](T x) { return bcv(u0, x); };
+    const V one = bc<V>(1.0), quarter = bc<V>(0.25), n1 = k(C.n1);
+    const V g2 = fma_(dx, dx, fma_(dy, dy, dz * dz));
+    const V rho = g2 + k(C.nx2);
+    const V iq = rsq(rho);
+    const V q = rho * iq;
+    const V irho = iq * iq;
+    V wp, wpk;              // W'(u) / wB K, W''(u) K
     if (C.well == 0) {
-        const F2 v = one - u0;
-        const F2 t = u0 * v;                                  // W' = 2 t (1 - 2u), W'' = 2 - 12 t
+        const V v = one - u0;
+        const V t = u0 * v;                                  // W' = 2 t (1 - 2u), W'' = 2 - 12 t
         wp = t * (v - u0);
-        wpk = fma_(t, dup(C.wA), dup(C.wB));
+        wpk = fma_(t, k(C.wA), k(C.wB));
     } else {
-        const F2 uu = u0 * u0;                                // W' = -u (1 - u^2), W'' = 3 u^2 - 1
+        const V uu = u0 * u0;                                // W' = -u (1 - u^2), W'' = 3 u^2 - 1
         wp = u0 * (one - uu);
-        wpk = fma_(uu, dup(C.wA), dup(C.wB));
+        wpk = fma_(uu, k(C.wA), k(C.wB));
     }
-    const F2 w = wp * dup(C.wB) * irho;
-    const F2 wx = w * dx, wy = w * dy, wz = w * dz;
-    const F2 Nxx = fma_(wx, dx, hxx), Nyy = fma_(wy, dy, hyy), Nzz = fma_(wz, dz, hzz);
-    const F2 Nxy = fma_(quarter, hxy, wx * dy), Nxz = fma_(quarter, hxz, wx * dz), Nyz = fma_(quarter, hyz, wy * dz);
-    const F2 Tr = Nxx + Nyy + Nzz;
-    const F2 off = fma_(Nxy, Nxy, fma_(Nxz, Nxz, Nyz * Nyz));
-    const F2 S = fma_(Nxx, Nxx, fma_(Nyy, Nyy, fma_(Nzz, Nzz, off + off)));
-    const F2 q4 = dup(C.n4) * q;
-    const F2 dT = fma_(dup(C.n2), Tr, q4);                    // half of de/dT
-    const F2 e = fma_(n1, S, fma_(Tr, dT + q4, dup(C.n6) * g2));
+    const V w = wp * k(C.wB) * irho;
+    const V wx = w * dx, wy = w * dy, wz = w * dz;
+    const V Nxx = fma_(wx, dx, hxx), Nyy = fma_(wy, dy, hyy), Nzz = fma_(wz, dz, hzz);
+    const V Nxy = fma_(quarter, hxy, wx * dy), Nxz = fma_(quarter, hxz, wx * dz), Nyz = fma_(quarter, hyz, wy * dz);
+    const V Tr = Nxx + Nyy + Nzz;
+    const V off = fma_(Nxy, Nxy, fma_(Nxz, Nxz, Nyz * Nyz));
+    const V S = fma_(Nxx, Nxx, fma_(Nyy, Nyy, fma_(Nzz, Nzz, off + off)));
+    const V q4 = k(C.n4) * q;
+    const V dT = fma_(k(C.n2), Tr, q4);                    // half of de/dT
+    const V e = fma_(n1, S, fma_(Tr, dT + q4, k(C.n6) * g2));
     if constexpr (!GRAD) return e;
-    const F2 Lxx = fma_(n1, Nxx, dT), Lyy = fma_(n1, Nyy, dT), Lzz = fma_(n1, Nzz, dT);
-    const F2 Lxy = n1 * Nxy, Lxz = n1 * Nxz, Lyz = n1 * Nyz;
-    const F2 LGx = fma_(Lxx, dx, fma_(Lxy, dy, Lxz * dz));
-    const F2 LGy = fma_(Lxy, dx, fma_(Lyy, dy, Lyz * dz));
-    const F2 LGz = fma_(Lxz, dx, fma_(Lyz, dy, Lzz * dz));
-    const F2 GLG = fma_(dx, LGx, fma_(dy, LGy, dz * LGz));
+    const V Lxx = fma_(n1, Nxx, dT), Lyy = fma_(n1, Nyy, dT), Lzz = fma_(n1, Nzz, dT);
+    const V Lxy = n1 * Nxy, Lxz = n1 * Nxz, Lyz = n1 * Nyz;
+    const V LGx = fma_(Lxx, dx, fma_(Lxy, dy, Lxz * dz));
+    const V LGy = fma_(Lxy, dx, fma_(Lyy, dy, Lyz * dz));
+    const V LGz = fma_(Lxz, dx, fma_(Lyz, dy, Lzz * dz));
+    const V GLG = fma_(dx, LGx, fma_(dy, LGy, dz * LGz));
     ct.u = wpk * GLG * irho;
-    const F2 al = w + w;
-    const F2 be = fma_(dup(C.n4) * Tr, iq, dup(C.n6)) - al * GLG * irho;
+    const V al = w + w;
+    const V be = fma_(k(C.n4) * Tr, iq, k(C.n6)) - al * GLG * irho;
     ct.dx = fma_(al, LGx, be * dx);
     ct.dy = fma_(al, LGy, be * dy);
     ct.dz = fma_(al, LGz, be * dz);

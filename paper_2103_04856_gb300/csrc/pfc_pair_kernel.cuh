@@ -44,6 +44,9 @@
 
 namespace pfc {
 
+constexpr int CBUF = 4;     // ring of coefficient planes (EXT = 2)
+constexpr int CP = 44;      // pitch of their rows: columns x0-4 .. x0+35
+
 template <int TY>
 struct PairTile {
     static constexpr int NPR = TY / 2 + 1;        // pair rows
@@ -56,7 +59,68 @@ struct PairTile {
     static constexpr int FP = 35;                 // pitch of a field pair row (34 columns and a guard column)
     static constexpr int FPL = (NPR + 2) * FP;    // one field plane, a guard row before and after
     static constexpr size_t SMEM = sizeof(F2) * ((size_t)NBUF * PLANE + 2 * 4 * FPL) + sizeof(float) * NPART * NT;
+    static constexpr int CR = TY + 2;             // rows of a coefficient plane: y0-1 .. y0+TY
+    static constexpr size_t CSMEM = sizeof(float) * (size_t)CBUF * NCF * CR * CP;   // EXT = 2
     static_assert(TY % 2 == 0 && 2 * NPR <= 32, "the halo columns' pairs fit one warp");
+};
+
+__device__ __forceinline__ void copy4(unsigned shared, const float* global)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(shared), "l"(global) : "memory");
+}
+
+__device__ __forceinline__ void copy16(unsigned shared, const float* global)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(shared), "l"(global) : "memory");
+}
+
+// The coefficients of one pair from its planes in shared memory (EXT = 2),
+// `plane` values each; c: the pair's first voxel.
+__device__ __forceinline__ void field_coefs(const float* c, int plane, Coef2& C)
+{
+    F2* const to[NCF] = { &C.c1, &C.c2, &C.c3, &C.c4, &C.c5, &C.c6 };
+#pragma unroll
+    for (int q = 0; q < NCF; ++q) *to[q] = pk(c[q * plane], c[q * plane + CP]);
+    C.c2x2 = C.c2 + C.c2;
+    C.c6x2 = C.c6 + C.c6;
+}
+
+// Copies of a run's coefficient planes (EXT = 2): rows yc .. yc + CR - 1,
+// columns x0 - 4 .. x0 + 35, periodic.  Rows of a multiple of four values go
+// in 16-byte pieces, one column of pieces for all six planes per thread;
+// others value by value, with the rows and columns of the u copies (rows r0
+// and r0 + 1 counted from yc, columns x0 - 2 .. x0 + 33).
+template <int CR>
+struct FieldCopy {
+    int off = -1;           // 16-byte path: this thread's piece in a plane, or -1
+    unsigned dst = 0;
+    __device__ __forceinline__ void init(int tid, int nx, int ny, int x0, int yc)
+    {
+        off = -1;
+        if (nx % 4 == 0 && tid < CR * 10) {
+            const int r = tid / 10, c = tid - r * 10;
+            off = wrapi(yc + r, ny) * nx + wrapi(x0 - 4 + 4 * c, nx);
+            dst = (unsigned)(r * CP + 4 * c) * 4;
+        }
+    }
+    __device__ __forceinline__ void issue(unsigned cs, const float* src, size_t stride, int nx, int lane, int r0, int offa,
+                                          int offb, int offc) const
+    {
+        if (nx % 4 == 0) {
+            if (off >= 0)
+#pragma unroll
+                for (int q = 0; q < NCF; ++q, src += stride) copy16(cs + dst + q * (CR * CP * 4), src + off);
+            return;
+        }
+        const bool a = r0 >= 0 && r0 < CR, b = r0 + 1 >= 0 && r0 + 1 < CR;
+        const unsigned d = cs + (unsigned)(r0 * CP + 2 + lane) * 4, e = cs + (unsigned)(r0 * CP + 34 + (lane & 3)) * 4;
+        for (int q = 0; q < NCF; ++q, src += stride) {
+            const unsigned o = (unsigned)q * (CR * CP * 4);
+            if (a) copy4(d + o, src + offa);
+            if (b) copy4(d + o + CP * 4, src + offb);
+            if (lane < 8 && ((lane & 4) ? b : a)) copy4(e + o + ((lane & 4) ? CP * 4 : 0), src + offc);
+        }
+    }
 };
 
 // A warp-uniform value, for the compiler to see as one (it then keeps what
@@ -81,7 +145,11 @@ __device__ __forceinline__ long long unit_at(const Launch<float, MAXI>& L, long 
     return in.unit_base + (rel < wf ? rel / in.w_full : nfull + (rel - wf) / in.w_last);
 }
 
-template <int TY, int MODE, int MAXI, bool SYM, bool HALO>
+// EXT: 1 = the orientation term of Sec. 5.2 (its weight c7 may be zero); 2 =
+// the same with coefficients read per voxel from a field c(x), whose six
+// planes travel through shared memory beside u's (24 more bytes a voxel-step):
+// held one plane ahead in registers they would not fit.
+template <int TY, int MODE, int MAXI, bool SYM, bool HALO, int EXT = 0>
 __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_constant__ Launch<float, MAXI> L)
 {
     using TL = PairTile<TY>;
@@ -90,6 +158,7 @@ __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_const
     F2* us = reinterpret_cast<F2*>(smem_raw);                   // [NBUF][UPR][UP]
     F2* fs = us + NBUF * PLANE;                                 // [2][4][NPR + 2][FP]
     float* scr = reinterpret_cast<float*>(fs + 2 * 4 * FPL);    // [NPART][NT]
+    float* cs = scr + NPART * NT;                               // EXT = 2: [CBUF][NCF][CR][CP]
     __shared__ double tot[NPART];
     __shared__ long long st[3];                   // the CTA's next unit, the end of its units, the next problem
 
@@ -177,21 +246,33 @@ __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_const
         const unsigned dstc = (unsigned)__cvta_generic_to_shared(us) + (warp * UP + 32 + (lane & 3)) * 8 +
                               ((lane & 4) ? UP * 8 : 4);
         int pz = wrapi(z0 - 2, nz);                    // planes are issued in increasing order
+        int pc = wrapi(z0 - 3, nz);                    // the plane before
+        const unsigned cso = (unsigned)__cvta_generic_to_shared(cs);
+        FieldCopy<TL::CR> fcopy;
+        if constexpr (EXT == 2) fcopy.init(tid, nx, ny, x0, y0 - 1);
         auto issue = [&](int p) {
             if (p <= plast) {
                 const unsigned o = (unsigned)(p & (NBUF - 1)) * (PLANE * 8);
                 const float* src = (HALO && (p < 0 || p >= nz)) ? in.halo + (size_t)(p < 0 ? p + 2 : p - nz + 2) * plane_g
                                                                 : in.u + (size_t)pz * plane_g;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dsta + o), "l"(src + offa) : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dsta + o + (UP * 8 - 4)), "l"(src + offb) : "memory");
+                copy4(dsta + o, src + offa);
+                copy4(dsta + o + (UP * 8 - 4), src + offb);
                 if (lane < 8)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dstc + o), "l"(src + offc) : "memory");
+                    copy4(dstc + o, src + offc);
+            }
+            if constexpr (EXT == 2) {   // the coefficients of plane p - 1
+                if (p >= z0 && p <= zend + 1)
+                    fcopy.issue(cso + (unsigned)((p - 1) & (CBUF - 1)) * (NCF * TL::CR * CP * 4),
+                                in.cf + (size_t)pc * plane_g, plane_g * nz, nx, lane, 2 * warp - 1, offa, offb, offc);
+                pc = pz;
             }
             cp_async_commit();   // one group per plane slot, empty past the run
             pz = pz + 1 == nz ? 0 : pz + 1;
         };
 
 #if PFC_DEBUG
+        if constexpr (EXT == 2)
+            for (int i = tid; i < CBUF * NCF * TL::CR * CP; i += NT) cs[i] = NAN;
         for (int i = tid; i < NBUF * PLANE + 2 * 4 * FPL; i += NT) {
             const int f = i - NBUF * PLANE, r = f < 0 ? 1 : (f % FPL) / FP;
             if (r > 0 && r <= NPR) us[i] = dup(NAN);
@@ -307,8 +388,12 @@ __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_const
                 };
                 Cot2 t;
                 F2 e;
-                if constexpr (SYM) e = pair_eval_sym<true>(C, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t);
-                else e = pair_eval<true>(C2, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t, refine);
+                if constexpr (SYM) e = eval_sym<true>(C, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t);
+                else {
+                    Coef2 Cv = C2;
+                    if constexpr (EXT == 2) field_coefs(cs + (m & (CBUF - 1)) * (NCF * TL::CR * CP) + 2 * pj * CP + ex + 3, TL::CR * CP, Cv);
+                    e = pair_eval<true, EXT != 0>(Cv, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t, refine);
+                }
                 if constexpr (kOwn) se = fma_(wI, e, se);
                 // transposed-stencil pieces of the pair (see the gather)
                 F2 X1, X2, Y1, Y2, zd, zu;
@@ -375,9 +460,11 @@ constexpr int PE_TY = 24;
 struct PairEnergyTile {
     static constexpr int NPR = PE_TY / 2, NW = NPR + 1, NT = NW * 32, UP = 37, PLANE = (NPR + 2) * UP;
     static constexpr size_t SMEM = sizeof(F2) * (size_t)NBUF * PLANE + sizeof(float) * NPART * NT;
+    static constexpr int CR = PE_TY;
+    static constexpr size_t CSMEM = sizeof(float) * (size_t)CBUF * NCF * CR * CP;
 };
 
-template <bool SYM, bool HALO>
+template <bool SYM, bool HALO, int EXT = 0>
 __global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __grid_constant__ Launch<float, 1> L)
 {
     using TL = PairEnergyTile;
@@ -385,6 +472,7 @@ __global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __g
     extern __shared__ __align__(16) unsigned char smem_raw[];
     F2* us = reinterpret_cast<F2*>(smem_raw);
     float* scr = reinterpret_cast<float*>(us + NBUF * PLANE);
+    float* cs = scr + NPART * NT;
     __shared__ double tot[NPART];
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const Inst<float>& in = L.inst[0];
@@ -416,16 +504,25 @@ __global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __g
         const unsigned dsta = (unsigned)__cvta_generic_to_shared(us) + (warp * UP + lane) * 8 + 4;
         const unsigned dstc = (unsigned)__cvta_generic_to_shared(us) + (warp * UP + 32 + (lane & 3)) * 8 +
                               ((lane & 4) ? UP * 8 : 4);
-        int pz = wrapi(z0 - 1, nz);
+        int pz = wrapi(z0 - 1, nz), pc = wrapi(z0 - 2, nz);
+        const unsigned cso = (unsigned)__cvta_generic_to_shared(cs);
+        FieldCopy<TL::CR> fcopy;
+        if constexpr (EXT == 2) fcopy.init(threadIdx.x, nx, ny, x0, y0);
         auto issue = [&](int p) {
             if (p <= zend) {
                 const unsigned o = (unsigned)(p & (NBUF - 1)) * (PLANE * 8);
                 const float* src = (HALO && (p < 0 || p >= nz)) ? in.halo + (size_t)(p < 0 ? p + 2 : p - nz + 2) * plane_g
                                                                 : in.u + (size_t)pz * plane_g;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dsta + o), "l"(src + offa) : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dsta + o + (UP * 8 - 4)), "l"(src + offb) : "memory");
+                copy4(dsta + o, src + offa);
+                copy4(dsta + o + (UP * 8 - 4), src + offb);
                 if (lane < 8)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dstc + o), "l"(src + offc) : "memory");
+                    copy4(dstc + o, src + offc);
+            }
+            if constexpr (EXT == 2) {   // the coefficients of plane p - 1
+                if (p > z0 && p <= zend)
+                    fcopy.issue(cso + (unsigned)((p - 1) & (CBUF - 1)) * (NCF * TL::CR * CP * 4),
+                                in.cf + (size_t)pc * plane_g, plane_g * nz, nx, lane, 2 * warp - 1, offa, offb, offc);
+                pc = pz;
             }
             cp_async_commit();
             pz = pz + 1 == nz ? 0 : pz + 1;
@@ -482,8 +579,13 @@ __global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __g
             };
             Cot2 t;
             F2 e;
-            if constexpr (SYM) e = pair_eval_sym<false>(C, u0, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t);
-            else e = pair_eval<false>(C2, u0, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t, refine);
+            if constexpr (SYM) e = eval_sym<false>(C, u0, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t);
+            else {
+                Coef2 Cv = C2;
+                if constexpr (EXT == 2)
+                    field_coefs(cs + (m & (CBUF - 1)) * (NCF * TL::CR * CP) + 2 * warp * CP + lane + 4, TL::CR * CP, Cv);
+                e = pair_eval<false, EXT != 0>(Cv, u0, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, t, refine);
+            }
             se = fma_(wI, e, se);
         };
         plane(z0, std::true_type{});
@@ -543,37 +645,44 @@ static void plan_pair(Launch<float, MAXI>& L, int TY, bool energy, int max_run)
     }
 }
 
-template <int TY, int MODE, int MAXI, bool SYM, bool HALO>
+template <int TY, int MODE, int MAXI, bool SYM, bool HALO, int EXT = 0>
 static cudaError_t launch_pair_one(Launch<float, MAXI>& L, int max_run, cudaStream_t s)
 {
     plan_pair(L, TY, false, max_run);
-    static bool attr_done = false;
+    const size_t smem = PairTile<TY>::SMEM + (EXT == 2 ? PairTile<TY>::CSMEM : 0);
+    static bool attr_done = false;   // idempotent, so a race between threads is harmless
     if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k_pair<TY, MODE, MAXI, SYM, HALO>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairTile<TY>::SMEM);
+        cudaError_t e = cudaFuncSetAttribute(k_pair<TY, MODE, MAXI, SYM, HALO, EXT>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    k_pair<TY, MODE, MAXI, SYM, HALO><<<L.grid, PairTile<TY>::NT, PairTile<TY>::SMEM, s>>>(L);
+    k_pair<TY, MODE, MAXI, SYM, HALO, EXT><<<L.grid, PairTile<TY>::NT, smem, s>>>(L);
     return cudaGetLastError();
 }
 
+template <bool SYM, bool HALO, int EXT = 0>
+static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStream_t s)
+{
+    plan_pair(L, PE_TY, true, max_run);
+    const size_t smem = PairEnergyTile::SMEM + (EXT == 2 ? PairEnergyTile::CSMEM : 0);
+    static bool attr_done = false;
+    if (!attr_done) {
+        cudaError_t e = cudaFuncSetAttribute(k_pair_energy<SYM, HALO, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_done = true;
+    }
+    k_pair_energy<SYM, HALO, EXT><<<L.grid, PairEnergyTile::NT, smem, s>>>(L);
+    return cudaGetLastError();
+}
+
+// tile_y: the height hint (pfc_problem.tile_y: 8, 13 or 16)
 template <int MAXI, bool SYM, bool HALO>
 static cudaError_t launch_pair_mode(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s)
 {
     if constexpr (MAXI == 1) {
-        if (mode == MODE_ENERGY) {
-            plan_pair(L, PE_TY, true, max_run);
-            static bool attr_done = false;
-            if (!attr_done) {
-                cudaError_t e = cudaFuncSetAttribute(k_pair_energy<SYM, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)PairEnergyTile::SMEM);
-                if (e != cudaSuccess) return e;
-                attr_done = true;
-            }
-            k_pair_energy<SYM, HALO><<<L.grid, PairEnergyTile::NT, PairEnergyTile::SMEM, s>>>(L);
-            return cudaGetLastError();
-        }
+        if (mode == MODE_ENERGY) return launch_pair_energy<SYM, HALO>(L, max_run, s);
     }
     const int rows = pair_tile_rows(tile_y);
     if (mode == MODE_GRAD)
@@ -585,6 +694,18 @@ static cudaError_t launch_pair_mode(Launch<float, MAXI>& L, int mode, int tile_y
                : rows == 12 ? launch_pair_one<12, MODE_STEP, MAXI, SYM, HALO>(L, max_run, s)
                             : launch_pair_one<20, MODE_STEP, MAXI, SYM, HALO>(L, max_run, s);
     return cudaErrorInvalidValue;
+}
+
+// The orientation term (EXT = 1) or a coefficient field (2): 20-row tiles.
+template <bool HALO, int EXT>
+static cudaError_t launch_pair_ext_mode(Launch<float, 1>& L, int mode, int max_run, cudaStream_t s)
+{
+    switch (mode) {
+    case MODE_ENERGY: return launch_pair_energy<false, HALO, EXT>(L, max_run, s);
+    case MODE_GRAD: return launch_pair_one<20, MODE_GRAD, 1, false, HALO, EXT>(L, max_run, s);
+    case MODE_STEP: return launch_pair_one<20, MODE_STEP, 1, false, HALO, EXT>(L, max_run, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace pfc

@@ -100,3 +100,32 @@ def test_symmetric_constants_out_of_range_take_the_general_form():
     assert abs(E - Eo) <= 1e-4 * abs(Eo)
     assert np.linalg.norm(g.double().cpu().numpy() - go) <= 1e-3 * np.linalg.norm(go)
     ctx.close()
+
+
+@pytest.mark.parametrize("nx", [30, 31, 32, 36, 65, 100])
+@pytest.mark.parametrize("ny, nz", [(1, 3), (21, 2), (24, 5), (41, 40)])
+def test_packed_extended_sweep_edges(nx, ny, nz):
+    """Coefficients from a field with the orientation term: its planes travel in 16-byte pieces where
+    nx is a multiple of four, else value by value; tiles ragged in both directions."""
+    shape = (nz, ny, nx)
+    u = I.noise(shape, 0.3, 0.1, 7).astype(np.float32).astype(np.float64)
+    rng = np.random.default_rng(nx + ny)
+    base = np.array(GEN)[:, None, None, None]
+    af = (base * (1.0 + 0.3 * rng.standard_normal((6,) + shape))).astype(np.float32)
+    mu, theta = 0.7, (0.6, 0.0, 0.8)
+    op = {"a": GEN, "eps": 1.5, "h": 1.0, "xi": 1e-2, "well": 0, "mu": mu, "theta": theta, "a_field": af.astype(np.float64)}
+    Eo, go = oracle.energy_and_grad(u, op)
+    ctx = pfc.Context(pfc.Problem.from_shape(shape, eps=1.5, a=GEN, xi=1e-2, mu=mu, theta=theta))
+    ctx.set_coefficient_field(torch.tensor(af, device="cuda"))
+    ud = torch.tensor(u, dtype=torch.float32, device="cuda")
+    E, g = ctx.energy_and_grad(ud)
+    gmax = np.abs(go).max()
+    assert abs(E - Eo) <= 1e-5 * max(abs(Eo), 1e-3 * u.size)
+    assert abs(ctx.energy(ud) - Eo) <= 1e-5 * max(abs(Eo), 1e-3 * u.size)
+    assert np.abs(g.double().cpu().numpy() - go).max() <= 1e-4 * gmax + 1e-7
+    out = torch.empty_like(ud)
+    ctx.step(ud, out, TAU)
+    lam = go.mean()
+    assert np.abs(out.double().cpu().numpy() - (u - TAU * (go - lam))).max() <= 2.0 ** -23 + TAU * (1e-4 * gmax + 1e-7)
+    ctx.close()
+
