@@ -65,6 +65,7 @@ struct pfc_ctx {
     double* trace = nullptr;
     int trace_cap = 0;
     void* plain_mem = nullptr;       // 21 fields for the plain path
+    void* work = nullptr;            // small FP64 grids: cotangents (launch_split)
     void* cfield = nullptr;          // c(x) from pfc_set_coefficient_field (NCF fields)
     bool cf_on = false;
     double* dpart = nullptr;         // diagnostics: block partials, ticket, 5 results
@@ -168,6 +169,14 @@ static pfc_status check_dev_ptr(const pfc_ctx* c, const void* ptr, const char* n
     return PFC_OK;
 }
 
+// bytes of work space for evaluations as two kernels of nz planes of the
+// problem (extra: planes beyond them, for a slab), 0 where the sweep serves
+static size_t split_bytes(const pfc_problem* p, int nz, int extra)
+{
+    if (p->prec != PFC_FP64 || !split_fits(p->nx, p->ny, nz, p->tile_y, p->tile_z, p->mu, p->proj)) return 0;
+    return split_work((long)p->nx * p->ny * (nz + extra));
+}
+
 static void free_ctx_mem(pfc_ctx* c)
 {
     cudaFree(c->ping);
@@ -177,6 +186,7 @@ static void free_ctx_mem(pfc_ctx* c)
     cudaFree(c->trace);
     cudaFree(c->plain_mem);
     cudaFree(c->cfield);
+    cudaFree(c->work);
     cudaFree(c->dpart);
     cudaFree(c->dticket);
     cudaFree(c->dout);
@@ -214,6 +224,10 @@ extern "C" pfc_status pfc_create(const pfc_problem* prob, pfc_ctx** out)
               cudaMalloc((void**)&c->ints, sizeof(unsigned) * NINTS) == cudaSuccess &&
               cudaMalloc((void**)&c->scal, sizeof(double) * NSCAL) == cudaSuccess &&
               cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok && prob->impl == PFC_IMPL_FUSED) {
+        const size_t bytes = split_bytes(prob, prob->nz, 0);
+        if (bytes) ok = cudaMalloc(&c->work, bytes) == cudaSuccess;
+    }
     if (ok && prob->impl == PFC_IMPL_PLAIN)
         ok = cudaMalloc(&c->plain_mem, (size_t)c->esz * c->N * 21) == cudaSuccess;
     // cleared on the context's own stream (no device-wide wait, see ensure_trace)
@@ -258,6 +272,7 @@ static Inst<T> make_inst(const pfc_ctx* c, const void* u, void* out, double tau)
     in.nblocks = c->nblocks;
     in.C = make_coef<T>(P.a, P.h, P.eps, P.xi, P.well, P.mu, P.theta, P.proj, refine_of(P));
     in.cf = c->cf_on ? (const T*)c->cfield : nullptr;
+    in.work = (T*)c->work;
     in.tau = (T)tau;
     in.inv_N = 1.0 / (double)c->N;
     in.partials = c->partials;
@@ -644,6 +659,7 @@ struct pfc_slab {
     double* partials = nullptr;
     double* scal = nullptr;
     unsigned* ints = nullptr;
+    void* work = nullptr;   // small FP64 slabs: cotangents (launch_split)
     int last_mode = -1;     // mode of the last sweep: what pfc_slab_finish combines
 };
 
@@ -673,8 +689,11 @@ extern "C" pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32
     geometry(&local, device_sms(), &sl->tile_y, &zc, &tx, &ty, &cz);
     sl->nblocks = (int)fused_grid(fused_units(prob->nx, prob->ny, nz_local), prob->tile_z);
     const size_t bytes = sizeof(double) * ((size_t)NPART * sl->nblocks + NSCAL) + sizeof(unsigned) * NINTS;
-    if (cudaMalloc((void**)&sl->mem, bytes) != cudaSuccess) {
+    const size_t wbytes = split_bytes(prob, nz_local, 2);
+    if (cudaMalloc((void**)&sl->mem, bytes) != cudaSuccess ||
+        (wbytes && cudaMalloc(&sl->work, wbytes) != cudaSuccess)) {
         (void)cudaGetLastError();
+        cudaFree(sl->mem);
         delete sl;
         return fail(PFC_ENOMEM, "device allocation of %zu bytes failed", bytes);
     }
@@ -688,6 +707,7 @@ extern "C" pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32
         cudaError_t e = cudaGetLastError();
         if (s) cudaStreamDestroy(s);
         cudaFree(sl->mem);
+        cudaFree(sl->work);
         delete sl;
         return fail(PFC_ECUDA, "clearing the slab's scalars failed: %s", cudaGetErrorString(e));
     }
@@ -704,6 +724,7 @@ extern "C" void pfc_slab_destroy(pfc_slab* sl)
     cudaSetDevice(sl->device);
     cudaDeviceSynchronize();
     cudaFree(sl->mem);
+    cudaFree(sl->work);
     cudaSetDevice(prev);
     delete sl;
 }
@@ -725,6 +746,7 @@ static Inst<T> slab_inst(const pfc_slab* sl, const void* u, const void* halo, vo
     in.ints = sl->ints;
     in.scal = sl->scal;
     in.halo = (const T*)halo;
+    in.work = (T*)sl->work;
     in.sums_out = sums;
     return in;
 }

@@ -329,6 +329,7 @@ cudaError_t launch_fused(const Inst<T>& in, int mode, int tile_y, int max_run, c
         return in.C.nform ? launch_pair_sym<1>(L, mode, tile_y, max_run, s) : launch_pair<1>(L, mode, tile_y, max_run, s);
     } else {
         if (needs_ext(in)) return launch_mode<T, EXT_TILE_Y, 1>(in, mode, max_run, s);
+        if (in.work) return launch_split(in, mode, s);
         if (tile_y == 8) return launch_mode<T, 8>(in, mode, max_run, s);
         if (tile_y == 13) return launch_mode<T, 13>(in, mode, max_run, s);
         return launch_mode<T, 16>(in, mode, max_run, s);

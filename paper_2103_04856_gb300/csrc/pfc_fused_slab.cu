@@ -34,6 +34,7 @@ cudaError_t launch_fused_halo(const Inst<T>& in, int mode, int tile_y, int max_r
         return launch_pair_halo(L, mode, tile_y, max_run, s);
     } else {
         if (needs_ext(in)) return launch_halo_mode<T, EXT_TILE_Y, 1>(in, mode, max_run, s);
+        if (in.work) return launch_split(in, mode, s);
         if (tile_y == 8) return launch_halo_mode<T, 8, 0>(in, mode, max_run, s);
         if (tile_y == 13) return launch_halo_mode<T, 13, 0>(in, mode, max_run, s);
         return launch_halo_mode<T, 16, 0>(in, mode, max_run, s);

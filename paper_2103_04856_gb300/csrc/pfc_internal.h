@@ -99,6 +99,9 @@ struct Inst {
     // (the two planes below the slab, then the two above) read instead of
     // wrapping around z
     const T* halo;
+    // FP64: null, or split_work(N) bytes: the evaluation runs as two kernels
+    // (launch_split)
+    T* work;
     // null, or NPART doubles receiving this launch's FP64 sums for the
     // problem (the scalars are then set by a later combine over all slabs)
     double* sums_out;
@@ -162,6 +165,13 @@ long long fused_grid(long long units, int max_run);
 // launch of it never has more CTAs, hence partial slots, than
 // fused_grid(fused_units(...), max_run).
 long long fused_units(int nx, int ny, int nz);
+// FP64 evaluations without extensions as two kernels, cotangents to memory and
+// the adjoint from it (pfc_split.cu), of problems that bring in.work
+constexpr long SPLIT_MAX = 1L << 22;
+// whether a problem (its slab of nz planes) takes them: at most SPLIT_MAX voxels
+bool split_fits(int nx, int ny, int nz, int tile_y, int tile_z, double mu, int proj);
+size_t split_work(long n);   // bytes; a z-slab counts a plane more on either side
+cudaError_t launch_split(const Inst<double>& in, int mode, cudaStream_t s);
 // the packed FP32 sweep (pfc_pair*.cu): plans the launch's tiles for the
 // height hint tile_y and runs it; general and symmetric polynomials, z-slabs
 template <int MAXI>

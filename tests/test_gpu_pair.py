@@ -129,3 +129,29 @@ def test_packed_extended_sweep_edges(nx, ny, nz):
     assert np.abs(out.double().cpu().numpy() - (u - TAU * (go - lam))).max() <= 2.0 ** -23 + TAU * (1e-4 * gmax + 1e-7)
     ctx.close()
 
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (1, 2, 3), (2, 3, 5), (32, 32, 32), (5, 40, 36)])
+@pytest.mark.parametrize("a, well", [(SYM, 0), (SYM, 1), (GEN, 0), (GEN, 1)])
+def test_fp64_two_kernel_form(shape, a, well):
+    """The FP64 two-kernel evaluation against the oracle at 1e-10, and against the fused sweep (which an
+    explicit tile height selects)."""
+    u = I.noise(shape, 0.3, 0.1, 11)
+    op = {"a": a, "eps": 1.5, "h": 1.0, "xi": 1e-2, "well": well}
+    Eo, go = oracle.energy_and_grad(u, op)
+    uo, _ = oracle.step(u, op, TAU)
+    ud = torch.tensor(u, device="cuda")
+    scale = max(np.abs(go).max(), 1e-3)
+    res = []
+    for tile_y in (0, 8):
+        ctx = pfc.Context(pfc.Problem.from_shape(shape, eps=1.5, a=a, xi=1e-2, well=well, prec="fp64", tile_y=tile_y))
+        E, g = ctx.energy_and_grad(ud)
+        assert abs(E - Eo) <= 1e-10 * max(abs(Eo), 1e-6 * u.size)
+        assert abs(ctx.energy(ud) - Eo) <= 1e-10 * max(abs(Eo), 1e-6 * u.size)
+        assert np.abs(g.cpu().numpy() - go).max() <= 1e-10 * scale
+        out = torch.empty_like(ud)
+        sc = torch.zeros(5, dtype=torch.float64, device="cuda")
+        ctx.step(ud, out, TAU, sc)
+        assert np.abs(out.cpu().numpy() - uo).max() <= 1e-13
+        res.append(sc.cpu().numpy())
+        ctx.close()
+    assert np.abs(res[0] - res[1]).max() <= 1e-10 * max(abs(Eo), scale)
