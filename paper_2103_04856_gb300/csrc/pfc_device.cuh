@@ -572,6 +572,7 @@ __device__ void finish_problem(const Inst<T>& in, int slot, int mode, const doub
         for (int i = 0; i < NPART; ++i) in.sums_out[i] = s[i];
     } else {
         set_scalars(s, in.inv_N, mode, in.scal, in.ints, in.trace, in.trace_cap, retire);
+        if (in.e_host) *in.e_host = s[P_E];
     }
     __threadfence();
     in.ints[I_TICKET] = 0;   // ready for the next launch on this problem

@@ -105,6 +105,9 @@ struct Inst {
     // null, or NPART doubles receiving this launch's FP64 sums for the
     // problem (the scalars are then set by a later combine over all slabs)
     double* sums_out;
+    // null, or a place in mapped host memory that receives the energy too: a
+    // caller that waits for it reads it there without a copy
+    double* e_host;
 };
 
 // Problems of one fused launch, passed by value as a kernel parameter (the

@@ -119,6 +119,7 @@ __device__ __forceinline__ void finish_split(const Inst<double>& in, int mode, d
         for (int i = 0; i < NPART; ++i) in.sums_out[i] = s[i];
     } else {
         set_scalars(s, in.inv_N, mode, in.scal, in.ints, in.trace, in.trace_cap);
+        if (in.e_host) *in.e_host = s[P_E];
     }
     __threadfence();
     in.ints[I_TICKET] = 0;
