@@ -27,7 +27,7 @@
 // voxels (168 registers) hide less latency than twenty of one, so the square
 // root's softplus is branch-free (root_softplus) and the run bookkeeping lives
 // in shared memory (the general form spilled 240 bytes per thread with it in
-// registers).  Tiles of 20 rows: 12 and 8 rows ran 1.17 and 1.6 times longer
+// registers).  Tiles of 20 rows (28 for symmetric polynomials, see sym_tall): 12 and 8 rows ran 1.17 and 1.6 times longer
 // on a 512^3 field.  A phase per plane on an mbarrier, waited for two planes
 // later, instead of a barrier per plane was 19 % slower.
 // Against the one-voxel sweep before it (32 x 16 and 32 x 13 tiles): four
@@ -455,20 +455,24 @@ __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_const
 }
 
 // The energy alone: no halo cotangents, no gather.  Warp j holds the rows
-// 2j, 2j + 1 of a 32 x PE_TY tile, lane = x; one more warp only copies.
-constexpr int PE_TY = 24;
+// 2j, 2j + 1 of a 32 x TY tile, lane = x; one more warp only copies.  General
+// polynomials take 30 rows (16 warps of 128 registers; 24 rows: 300^3 170 ->
+// 161 us, 133 x 150 x 201 50 -> 48), symmetric ones 24, which measure the same
+// within 4 % either way.
+template <bool SYM>
 struct PairEnergyTile {
-    static constexpr int NPR = PE_TY / 2, NW = NPR + 1, NT = NW * 32, UP = 37, PLANE = (NPR + 2) * UP;
+    static constexpr int TY = SYM ? 24 : 30;
+    static constexpr int NPR = TY / 2, NW = NPR + 1, NT = NW * 32, UP = 37, PLANE = (NPR + 2) * UP;
     static constexpr size_t SMEM = sizeof(F2) * (size_t)NBUF * PLANE + sizeof(float) * NPART * NT;
-    static constexpr int CR = PE_TY;
+    static constexpr int CR = TY;
     static constexpr size_t CSMEM = sizeof(float) * (size_t)CBUF * NCF * CR * CP;
 };
 
 template <bool SYM, bool HALO, int EXT = 0>
-__global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __grid_constant__ Launch<float, 1> L)
+__global__ void __launch_bounds__(PairEnergyTile<SYM>::NT, 1) k_pair_energy(const __grid_constant__ Launch<float, 1> L)
 {
-    using TL = PairEnergyTile;
-    constexpr int NPR = TL::NPR, NT = TL::NT, UP = TL::UP, PLANE = TL::PLANE;
+    using TL = PairEnergyTile<SYM>;
+    constexpr int PE_TY = TL::TY, NPR = TL::NPR, NT = TL::NT, UP = TL::UP, PLANE = TL::PLANE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     F2* us = reinterpret_cast<F2*>(smem_raw);
     float* scr = reinterpret_cast<float*>(us + NBUF * PLANE);
@@ -609,6 +613,12 @@ __global__ void __launch_bounds__(PairEnergyTile::NT, 1) k_pair_energy(const __g
 // in proportion to the warps made the CTAs that hold ragged planes finish
 // last, a 512^3 step 27 % slower).  With few planes per CTA, or a cap on them,
 // every plane weighs the same.
+static inline int plane_cost(int rows, bool energy)
+{
+    const int r = (rows + 1) / 2;
+    return 16 + (energy ? r : r + 2 - rows % 2);
+}
+
 template <int MAXI>
 static void plan_pair(Launch<float, MAXI>& L, int TY, bool energy, int max_run)
 {
@@ -621,7 +631,7 @@ static void plan_pair(Launch<float, MAXI>& L, int TY, bool energy, int max_run)
         units += (long long)in.tiles_x * in.tiles_y * in.nz;
     }
     const bool weigh = max_run <= 0 && units > 4LL * device_sms();
-    auto cost = [&](int rows) { const int r = (rows + 1) / 2; return 16 + (energy ? r : r + 2 - rows % 2); };
+    auto cost = [&](int rows) { return plane_cost(rows, energy); };
     long long W = 0;
     for (int k = 0; k < L.n; ++k) {
         Inst<float>& in = L.inst[k];
@@ -645,6 +655,31 @@ static void plan_pair(Launch<float, MAXI>& L, int TY, bool energy, int max_run)
     }
 }
 
+// Symmetric polynomials fit 128 registers, so 16 warps and tiles of 28 rows (24
+// ran 5 % slower than 20: 14 warps share four schedulers unevenly).  A plane of
+// 28 rows takes 1.15 to 1.25 times what plan_pair's weights say of it against
+// one of 20 (measured on eleven grids of 64 to 333 rows), a few percent less a
+// row; which height is faster is then a matter of the ragged last row of tiles,
+// so the weights' sums are compared.  Gradients: 128 x 112 x 128 28.6 -> 27.0 us,
+// 150 x 333 x 129 79.5 -> 73.8, four 128^3 problems a step 93.8 -> 89.9; where 20
+// rows fit (100, 160, 200) 28 ones took 3 to 9 % longer.
+template <int MAXI>
+static bool sym_tall(const Launch<float, MAXI>& L)
+{
+    auto column = [](int ny, int TY) {
+        const int full = (ny - 1) / TY, last = ny - full * TY;
+        return full * plane_cost(TY, false) + plane_cost(last, false);
+    };
+    double w20 = 0, w28 = 0;
+    for (int k = 0; k < L.n; ++k) {
+        const Inst<float>& in = L.inst[k];
+        const double planes = (double)((in.nx + TX - 1) / TX) * in.nz;
+        w20 += planes * column(in.ny, 20);
+        w28 += planes * 1.21 * column(in.ny, 28);
+    }
+    return w28 < w20;
+}
+
 template <int TY, int MODE, int MAXI, bool SYM, bool HALO, int EXT = 0>
 static cudaError_t launch_pair_one(Launch<float, MAXI>& L, int max_run, cudaStream_t s)
 {
@@ -664,8 +699,9 @@ static cudaError_t launch_pair_one(Launch<float, MAXI>& L, int max_run, cudaStre
 template <bool SYM, bool HALO, int EXT = 0>
 static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStream_t s)
 {
-    plan_pair(L, PE_TY, true, max_run);
-    const size_t smem = PairEnergyTile::SMEM + (EXT == 2 ? PairEnergyTile::CSMEM : 0);
+    using TL = PairEnergyTile<SYM>;
+    plan_pair(L, TL::TY, true, max_run);
+    const size_t smem = TL::SMEM + (EXT == 2 ? TL::CSMEM : 0);
     static bool attr_done = false;
     if (!attr_done) {
         cudaError_t e = cudaFuncSetAttribute(k_pair_energy<SYM, HALO, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -673,7 +709,7 @@ static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStre
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    k_pair_energy<SYM, HALO, EXT><<<L.grid, PairEnergyTile::NT, smem, s>>>(L);
+    k_pair_energy<SYM, HALO, EXT><<<L.grid, TL::NT, smem, s>>>(L);
     return cudaGetLastError();
 }
 
@@ -685,6 +721,12 @@ static cudaError_t launch_pair_mode(Launch<float, MAXI>& L, int mode, int tile_y
         if (mode == MODE_ENERGY) return launch_pair_energy<SYM, HALO>(L, max_run, s);
     }
     const int rows = pair_tile_rows(tile_y);
+    if constexpr (SYM) {
+        if (rows == 20 && sym_tall(L))
+            return mode == MODE_GRAD   ? launch_pair_one<28, MODE_GRAD, MAXI, SYM, HALO>(L, max_run, s)
+                   : mode == MODE_STEP ? launch_pair_one<28, MODE_STEP, MAXI, SYM, HALO>(L, max_run, s)
+                                       : cudaErrorInvalidValue;
+    }
     if (mode == MODE_GRAD)
         return rows == 8    ? launch_pair_one<8, MODE_GRAD, MAXI, SYM, HALO>(L, max_run, s)
                : rows == 12 ? launch_pair_one<12, MODE_GRAD, MAXI, SYM, HALO>(L, max_run, s)

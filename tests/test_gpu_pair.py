@@ -155,3 +155,34 @@ def test_fp64_two_kernel_form(shape, a, well):
         res.append(sc.cpu().numpy())
         ctx.close()
     assert np.abs(res[0] - res[1]).max() <= 1e-10 * max(abs(Eo), scale)
+
+
+@pytest.mark.parametrize("shape", [(3, 21, 31), (1, 26, 33), (4, 27, 35), (2, 28, 64), (60, 55, 97), (64, 56, 130),
+                                   (70, 53, 65)])
+def test_packed_tall_tiles(shape):
+    """Heights at which symmetric polynomials take tiles of 28 rows (whole, and ragged by one to seven rows)."""
+    _cmp(shape, SYM, 0, 0)
+
+
+@pytest.mark.parametrize("a", [GEN, SYM])
+@pytest.mark.parametrize("shape", [(3, 29, 31), (2, 30, 33), (5, 31, 64), (40, 61, 97)])
+def test_packed_energy_tiles(shape, a):
+    """The energy alone: heights around its tiles of 30 rows."""
+    _cmp(shape, a, 1, 0)
+
+
+def test_packed_batch_with_tall_tiles():
+    """A batch of symmetric polynomials whose heights together ask for tiles of 28 rows: each as alone."""
+    shapes = [(30, 56, 37), (50, 28, 66), (9, 27, 129), (64, 20, 33)]
+    probs = [pfc.Problem.from_shape(s, eps=1.5, a=SYM, xi=1e-2, well=k % 2) for k, s in enumerate(shapes)]
+    us = [torch.tensor(I.noise(s, 0.3, 0.1, k), dtype=torch.float32, device="cuda") for k, s in enumerate(shapes)]
+    outs = [torch.empty_like(u) for u in us]
+    b = pfc.Batch(probs)
+    b.step(us, outs, TAU)
+    for p, u, o in zip(probs, us, outs):
+        alone = torch.empty_like(u)
+        ctx = pfc.Context(p)
+        ctx.step(u, alone, TAU)
+        assert (o - alone).abs().max().item() <= 2.0 ** -22
+        ctx.close()
+    b.close()
