@@ -260,10 +260,11 @@ extern "C" void pfc_destroy(pfc_ctx* c)
 }
 
 template <typename T>
-static Inst<T> make_inst(const pfc_ctx* c, const void* u, void* out, double tau, double* e_host)
+static Inst<T> make_inst(const pfc_ctx* c, const void* u, void* out, double tau, double* e_host, bool chained)
 {
     Inst<T> in{};
     in.e_host = e_host;
+    in.chained = chained;
     const pfc_problem& P = c->P;
     in.u = (const T*)u;
     in.out = (T*)out;
@@ -301,9 +302,10 @@ static PlainBufs<T> plain_bufs(const pfc_ctx* c)
 
 // Enqueue one evaluation (MODE_ENERGY / MODE_GRAD) or one step (MODE_STEP;
 // fused: lazy offset, plain: explicit projection).  e_host: null or c->e_host,
-// which the fused kernels then fill with the energy.
+// which the fused kernels then fill with the energy.  chained: what is before
+// on the stream is a step of the same call.
 static cudaError_t enqueue(pfc_ctx* c, int mode, const void* u, void* out, double tau, cudaStream_t s,
-                           double* e_host = nullptr)
+                           double* e_host = nullptr, bool chained = false)
 {
     if (c->P.impl == PFC_IMPL_PLAIN) {
         if (c->P.prec == PFC_FP64)
@@ -317,8 +319,8 @@ static cudaError_t enqueue(pfc_ctx* c, int mode, const void* u, void* out, doubl
                                    c->trace, c->trace_cap, s);
     }
     if (c->P.prec == PFC_FP64)
-        return launch_fused<double>(make_inst<double>(c, u, out, tau, e_host), mode, c->tile_y, c->P.tile_z, s);
-    return launch_fused<float>(make_inst<float>(c, u, out, tau, e_host), mode, c->tile_y, c->P.tile_z, s);
+        return launch_fused<double>(make_inst<double>(c, u, out, tau, e_host, chained), mode, c->tile_y, c->P.tile_z, s);
+    return launch_fused<float>(make_inst<float>(c, u, out, tau, e_host, chained), mode, c->tile_y, c->P.tile_z, s);
 }
 
 // Wait for the energy of the evaluation enqueued last: from mapped host memory
@@ -414,7 +416,7 @@ static cudaError_t enqueue_steps(pfc_ctx* c, void* a, void* b, int i0, int n, do
 {
     for (int i = i0; i < i0 + n; ++i) {
         const bool even = (i % 2) == 0;
-        cudaError_t e = enqueue(c, MODE_STEP, even ? a : b, even ? b : a, tau, s);
+        cudaError_t e = enqueue(c, MODE_STEP, even ? a : b, even ? b : a, tau, s, nullptr, i > i0);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

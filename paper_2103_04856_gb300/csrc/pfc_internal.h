@@ -108,6 +108,9 @@ struct Inst {
     // null, or a place in mapped host memory that receives the energy too: a
     // caller that waits for it reads it there without a copy
     double* e_host;
+    // FP64 as two kernels: 1 if what is before on the stream is a step of the
+    // same call (launch_chained)
+    int chained;
 };
 
 // Problems of one fused launch, passed by value as a kernel parameter (the

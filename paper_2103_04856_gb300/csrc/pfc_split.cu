@@ -10,7 +10,9 @@
 // on a 32^3 grid (runs of one plane, 11 warps for 8 rows) is every voxel four
 // times, and always takes the softplus's exp and log1p (about 150 operations),
 // also where its weight is zero.  Here symmetric polynomials leave them out
-// and every voxel is evaluated once: a 32^3 step 79 -> 22 us.
+// and every voxel is evaluated once: a 32^3 step 79 -> 22 us, 20.5 with the
+// next kernel's blocks waiting on the SMs (pfc_chain.cuh).
+#include "pfc_chain.cuh"
 #include "pfc_pair.cuh"
 
 namespace pfc {
@@ -133,9 +135,11 @@ __device__ __forceinline__ double* split_part(double* F, int n) { return F + (lo
 // HALO (a z-slab): the n voxels are those of its planes and of one more on
 // either side, whose u comes from in.halo and whose density is not counted.
 template <bool SYM, bool GRAD, bool HALO>
-__global__ void __launch_bounds__(kThreads) k_cot(const __grid_constant__ Inst<double> in, int n, int mode, double* __restrict__ F)
+__global__ void __launch_bounds__(kThreads) k_cot(const __grid_constant__ Inst<double> in, int n, int mode, double* __restrict__ F_)
 {
-    const double* __restrict__ u = in.u;
+    chain_wait();
+    const double* __restrict__ u = after_wait(in.u);
+    double* __restrict__ F = after_wait(F_);
     const double c = mode == MODE_STEP ? in.scal[S_C] : 0.0;
     const Coef<double>& C = in.C;
     const int nz = in.nz;
@@ -196,8 +200,10 @@ __global__ void __launch_bounds__(kThreads) k_cot(const __grid_constant__ Inst<d
 }
 
 template <bool SYM, int MODE, bool HALO>
-__global__ void __launch_bounds__(kThreads) k_adj(const __grid_constant__ Inst<double> in, int n, double* __restrict__ F)
+__global__ void __launch_bounds__(kThreads) k_adj(const __grid_constant__ Inst<double> in, int n, double* __restrict__ F_)
 {
+    chain_wait();
+    double* __restrict__ F = after_wait(F_);
     const double c = MODE == MODE_STEP ? in.scal[S_C] : 0.0;
     double* part = split_part(F, n);
     double v[NPART] = { 0, 0, 0, 0, 0, 0 };
@@ -259,12 +265,12 @@ static void split(const Inst<double>& in, int mode, cudaStream_t s)
     const long n = (long)in.nx * in.ny * (in.nz + (HALO ? 2 : 0));
     const int nb = split_blocks(n);
     if (mode == MODE_ENERGY) {
-        k_cot<SYM, false, HALO><<<nb, kThreads, 0, s>>>(in, (int)n, mode, in.work);
+        launch_chained(in.chained != 0, k_cot<SYM, false, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
         return;
     }
-    k_cot<SYM, true, HALO><<<nb, kThreads, 0, s>>>(in, (int)n, mode, in.work);
-    if (mode == MODE_GRAD) k_adj<SYM, MODE_GRAD, HALO><<<nb, kThreads, 0, s>>>(in, (int)n, in.work);
-    else k_adj<SYM, MODE_STEP, HALO><<<nb, kThreads, 0, s>>>(in, (int)n, in.work);
+    launch_chained(in.chained != 0, k_cot<SYM, true, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
+    if (mode == MODE_GRAD) launch_chained(true, k_adj<SYM, MODE_GRAD, HALO>, nb, kThreads, 0, s, in, (int)n, in.work);
+    else launch_chained(true, k_adj<SYM, MODE_STEP, HALO>, nb, kThreads, 0, s, in, (int)n, in.work);
 }
 
 cudaError_t launch_split(const Inst<double>& in, int mode, cudaStream_t s)
