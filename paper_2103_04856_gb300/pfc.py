@@ -712,9 +712,9 @@ class PhaseFieldEnergy(torch.autograd.Function):
     def forward(fctx, u, ctx: Context):
         E, g = ctx.energy_and_grad(u.detach().contiguous())
         fctx.save_for_backward(g)
-        return torch.tensor(E, dtype=torch.float64, device=u.device)
+        return torch.full((), E, dtype=torch.float64, device=u.device)   # a kernel, not a copy and its wait
 
     @staticmethod
     def backward(fctx, grad_out):
         (g,) = fctx.saved_tensors
-        return (grad_out.to(g.dtype) * g), None
+        return torch.mul(g, grad_out), None      # of g's dtype: grad_out has no dimensions
