@@ -31,10 +31,10 @@
 // on a 512^3 field.  A phase per plane on an mbarrier, waited for two planes
 // later, instead of a barrier per plane was 19 % slower.
 // Against the one-voxel sweep before it (32 x 16 and 32 x 13 tiles): four
-// symmetric 128^3 problems 92 -> 84 us a launch, a 512^3 general step 1.82 ->
+// symmetric 128^3 problems 92 -> 80 us a launch, a 512^3 general step 1.82 ->
 // 1.64 ms, a 256^3 general step at xi = 1e-2 0.251 -> 0.211 ms, 24 mixed
 // problems 0.413 -> 0.341 ms a step, the energy of 201 x 150 x 133 voxels 112
-// -> 62 us, a 150-odd^3 step with rows of no multiple of four 264 -> 163 us.
+// -> 51 us, a 150-odd^3 step with rows of no multiple of four 264 -> 163 us.
 #pragma once
 
 #include <type_traits>
