@@ -173,7 +173,9 @@ pfc_status pfc_surface_cells(pfc_ctx* ctx, const void* u, double level, void* ce
  * sums the areas of the cells whose kappa1 falls in bin b1 and kappa2 in bin
  * b2 of [lo, hi) split in nbins; values outside are clamped into the edge bins
  * (the paper truncates its diagrams to [-100, 100]).  FP64 atomics: the sums
- * are exact up to rounding order.  Enqueue only. */
+ * are exact up to rounding order.  Enqueue only, on any stream; a call with
+ * many cells takes up to 16 MB of scratch in the order of the stream, from a
+ * pool of which the context keeps 32 MB (a captured call takes none). */
 pfc_status pfc_curvature_histogram(pfc_ctx* ctx, const void* cells, int64_t n, int32_t nbins, double lo,
                                    double hi, double* hist_dev, pfc_stream stream);
 

@@ -75,8 +75,7 @@ struct pfc_ctx {
     void* skap = nullptr;            // surface cells: kappa1, kappa2 fields, counts and masks, offsets
     unsigned* sblk = nullptr;
     long long* soff = nullptr;
-    double* hpart = nullptr;         // curvature histogram: hcap doubles of partial tables
-    size_t hcap = 0;
+    cudaMemPool_t hpool = nullptr;   // curvature histogram: the tables of calls under way
     // cached step-loop graph
     cudaGraphExec_t gexec = nullptr;
     const void* g_u = nullptr;
@@ -195,7 +194,7 @@ static void free_ctx_mem(pfc_ctx* c)
     cudaFree(c->skap);
     cudaFree(c->sblk);
     cudaFree(c->soff);
-    cudaFree(c->hpart);
+    if (c->hpool) cudaMemPoolDestroy(c->hpool);
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->cap) cudaStreamDestroy(c->cap);
 }
@@ -619,6 +618,50 @@ extern "C" pfc_status pfc_surface_cells(pfc_ctx* c, const void* u, double level,
     return PFC_OK;
 }
 
+// Tables for one histogram, in the order of the stream: this call's own, from
+// its launches to the cudaFreeAsync behind them, so that calls on several
+// streams do not meet and nothing waits.  The context's pool keeps what comes
+// back (kHistPool bytes) for the next call: mapping it anew takes longer than
+// the histogram.  Null where one table serves, where the stream is being
+// captured (a graph must not hold memory that the context owns) and where no
+// memory is left: the histogram then adds into hist_dev directly.
+constexpr unsigned long long kHistPool = 32ull << 20;
+static double* histogram_tables(pfc_ctx* c, long long n, int nbins, cudaStream_t s)
+{
+    const int copies = histogram_copies(n, nbins);
+    if (copies == 1) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (!c->hpool) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = c->device;
+        unsigned long long keep = kHistPool;
+        // relaxed: a capture under way on another stream does not mind a new pool
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        bool ok = cudaMemPoolCreate(&c->hpool, &props) == cudaSuccess;
+        ok = ok && cudaMemPoolSetAttribute(c->hpool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!ok) {
+            if (c->hpool) cudaMemPoolDestroy(c->hpool);
+            c->hpool = nullptr;
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+    }
+    void* part = nullptr;
+    if (cudaMallocFromPoolAsync(&part, sizeof(double) * (size_t)copies * nbins * nbins, c->hpool, s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return (double*)part;
+}
+
 extern "C" pfc_status pfc_curvature_histogram(pfc_ctx* c, const void* cells, int64_t n, int32_t nbins, double lo,
                                               double hi, double* hist_dev, pfc_stream stream)
 {
@@ -629,21 +672,15 @@ extern "C" pfc_status pfc_curvature_histogram(pfc_ctx* c, const void* cells, int
     if (st) return st;
     if (n > 0 && (st = check_dev_ptr(c, cells, "cells"))) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int copies = histogram_copies(nbins);
-    const size_t need = copies > 1 ? (size_t)copies * nbins * nbins : 0;
-    if (need > c->hcap) {   // grown only: at most 16 MB
-        PFC_CU(cudaStreamSynchronize(s));
-        cudaFree(c->hpart);
-        c->hpart = nullptr;
-        c->hcap = 0;
-        PFC_CU(cudaMalloc((void**)&c->hpart, sizeof(double) * need));
-        c->hcap = need;
+    double* part = histogram_tables(c, n, nbins, s);
+    cudaError_t e = c->P.prec == PFC_FP64
+                        ? launch_curvature_histogram<double>((const double*)cells, n, nbins, lo, hi, part, hist_dev, s)
+                        : launch_curvature_histogram<float>((const float*)cells, n, nbins, lo, hi, part, hist_dev, s);
+    if (part) {
+        const cudaError_t f = cudaFreeAsync(part, s);
+        if (e == cudaSuccess) e = f;
     }
-    double* part = need ? c->hpart : nullptr;
-    if (c->P.prec == PFC_FP64)
-        PFC_CU(launch_curvature_histogram<double>((const double*)cells, n, nbins, lo, hi, part, hist_dev, s));
-    else
-        PFC_CU(launch_curvature_histogram<float>((const float*)cells, n, nbins, lo, hi, part, hist_dev, s));
+    PFC_CU(e);
     return PFC_OK;
 }
 

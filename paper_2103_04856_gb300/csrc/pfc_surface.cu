@@ -344,8 +344,8 @@ __device__ __forceinline__ int hist_bin(float x, double lo, double inv_w, float 
 // Area-weighted 2-D histogram of (kappa1, kappa2) over [lo, hi)^2, values
 // outside clamped into the edge bins; hist[b1 * nbins + b2] (FP64 atomics).
 // Curvatures crowd into few bins, and atomics on one address queue in L2 (790
-// us for 4.4 million cells in one table), so the blocks spread over `copies`
-// tables (44 us), which k_hist_sum adds up (8 us).
+// us for 4.4 million cells in one table), so with many cells the blocks spread
+// over `copies` tables (44 us), which k_hist_sum adds up (8 us).
 template <typename T>
 __global__ void k_curv_hist(const T* __restrict__ cells, long long n, int nbins, double lo, double inv_w, int copies,
                             double* __restrict__ hist)
@@ -428,9 +428,14 @@ template cudaError_t launch_surface_cells<float>(const float*, const float*, con
 template cudaError_t launch_surface_cells<double>(const double*, const double*, const double*, int, int, int, double,
                                                   double, unsigned*, long long*, double*, long long, cudaStream_t);
 
-// Tables of the histogram: one per SM while they take no more than 16 MB.
-int histogram_copies(int nbins)
+// Tables of the histogram: one per SM while they take no more than 16 MB.  Few
+// cells for the bins add into one: its atomics take about 10 ns times n / nbins
+// (20 to 700 bins of smooth surfaces; noise a little less above 100 bins), and
+// the tables' own scratch, clearing and sum make a call 24 us instead of 16.
+// 100 bins: 110 000 cells 18 us (24 in tables), 240 000 29 (25), 7.2 million 725 (69).
+int histogram_copies(long long n, int nbins)
 {
+    if (n < 1600LL * nbins) return 1;
     const double bytes = 8.0 * nbins * nbins;
     const double c = 16.0 * 1024 * 1024 / bytes;
     return c < 2.0 ? 1 : (c < device_sms() ? (int)c : device_sms());
@@ -441,7 +446,7 @@ cudaError_t launch_curvature_histogram(const T* cells, long long n, int nbins, d
                                        double* hist, cudaStream_t s)
 {
     const long bins = (long)nbins * nbins;
-    const int copies = part ? histogram_copies(nbins) : 1;
+    const int copies = part ? histogram_copies(n, nbins) : 1;
     double* to = copies > 1 ? part : hist;
     cudaError_t e = cudaMemsetAsync(to, 0, sizeof(double) * (size_t)bins * copies, s);
     if (e != cudaSuccess) return e;
