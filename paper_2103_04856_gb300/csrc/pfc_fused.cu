@@ -225,7 +225,9 @@ Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, 
     auto fits = [](double v) { return v == 0.0 || (fabs(v) > 1e-30 && fabs(v) < 1e30); };
     C.nform = C.sym && n[4] > 1e-30;
     for (double v : n) C.nform = C.nform && fits(v);
-    C.nform = C.nform && fits(K);
+    // eval_sym's N is up to |K| W', its square is summed, and w up to |K| W' / nx2
+    // on a flat voxel: below 1e30 for W' of order 1, with room for larger u
+    C.nform = C.nform && fits(K) && fabs(K) < 1e15 && fabs(K) < 1e30 * n[4];
     return C;
 }
 template Coef<float> make_coef<float>(const double*, double, double, double, int, double, const double*, int, int);

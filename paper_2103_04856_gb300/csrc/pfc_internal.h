@@ -61,7 +61,8 @@ struct Coef {
     // 0/1: wA = -12 K, wB = 2 K; wells -1/1: wA = 3 K, wB = -K
     T wA, wB;
     // c1 kd^2, c2 kd^2, c4 sg kd / 2, c6 sg^2, xi^2 / sg^2; nform: sym, and all
-    // of them are representable (else the general form runs)
+    // of them and what they are multiplied to are representable (else the
+    // general form runs)
     T n1, n2, n4, n6, nx2;
     int nform;
 };
