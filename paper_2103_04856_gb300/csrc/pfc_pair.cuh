@@ -10,6 +10,7 @@
 #pragma once
 
 #include "pfc_device.cuh"
+#include "pfc_log1p.h"
 
 namespace pfc {
 
@@ -81,9 +82,11 @@ __device__ __forceinline__ F2 rsq(F2 a) { return pk(rsqrtf(lo(a)), rsqrtf(hi(a))
 __device__ __forceinline__ double rsq(double a) { return rsqrt(a); }
 
 // Coefficients of eq. Feps and the stencil scales as pairs, for the general
-// form, formed once per run.
+// form, formed once per run (2 c2 is not: without its registers the batched
+// step spills 80/148 bytes a thread instead of 124/192, 24 mixed problems
+// 5.8 -> 5.5 ms for 16 steps).
 struct Coef2 {
-    F2 c1, c2, c3, c4, c5, c6, c2x2, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
+    F2 c1, c2, c3, c4, c5, c6, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
     F2 c7, c7x2, th0, th1, th2;       // orientation term (ORIENT)
     float xi, xi64, inv_xi, rthr;
     int well;
@@ -92,7 +95,7 @@ __device__ __forceinline__ Coef2 coef2(const Coef<float>& C)
 {
     Coef2 P;
     P.c1 = dup(C.c1); P.c2 = dup(C.c2); P.c3 = dup(C.c3); P.c4 = dup(C.c4); P.c5 = dup(C.c5); P.c6 = dup(C.c6);
-    P.c2x2 = dup(C.c2x2); P.c6x2 = dup(C.c6x2);
+    P.c6x2 = dup(C.c6x2);
     P.c7 = dup(C.c7); P.c7x2 = dup(2.0f * C.c7); P.th0 = dup(C.th0); P.th1 = dup(C.th1); P.th2 = dup(C.th2);
     P.kd = dup(C.kd); P.ko = dup(C.ko); P.ko2 = dup(C.ko2); P.sg = dup(C.sg); P.nsg = dup(-C.sg);
     P.ie = dup(C.inv_eps); P.xi2 = dup(C.xi2);
@@ -108,22 +111,11 @@ __device__ __forceinline__ float ex2_(float x)
     return r;
 }
 
-// log(1 + x) for x in [0, 1]: x times a degree-9 minimax fit of log(1 + x) / x
-// (reweighted least squares in Chebyshev polynomials on [0, 1], relative error
-// 4.7e-9; with FP32 rounding at most 1.5e-7).
-__device__ __forceinline__ F2 log1p01(F2 x)
-{
-    F2 p = fma_(dup(-3.244023304e-03f), x, dup(1.985145360e-02f));
-    p = fma_(p, x, dup(-5.695951730e-02f));
-    p = fma_(p, x, dup(1.060365364e-01f));
-    p = fma_(p, x, dup(-1.530559212e-01f));
-    p = fma_(p, x, dup(1.967593879e-01f));
-    p = fma_(p, x, dup(-2.495413423e-01f));
-    p = fma_(p, x, dup(3.332996368e-01f));
-    p = fma_(p, x, dup(-4.999990165e-01f));
-    p = fma_(p, x, dup(1.0f));
-    return p * x;
-}
+struct PairArith {   // for log1p01
+    using V = F2;
+    static __device__ __forceinline__ F2 c(float x) { return dup(x); }
+    static __device__ __forceinline__ F2 fma(F2 a, F2 b, F2 x) { return fma_(a, b, x); }
+};
 
 // sqrt(P(D)) and d sqrt(P) / dD of both voxels (softplus_, one reciprocal
 // square root for both; 0 where P underflows to 0), without branches: where
@@ -138,7 +130,7 @@ __device__ __forceinline__ void root_softplus(float D0, float D1, const Coef2& C
     const F2 ex = pk(e0, e1), den = ex + dup(1.0f);
     const F2 inv = pk(__fdividef(1.0f, lo(den)), __fdividef(1.0f, hi(den)));
     const F2 exi = ex * inv;
-    const F2 P = fma_(dup(C.xi), log1p01(ex), pk(fmaxf(D0, 0.0f), fmaxf(D1, 0.0f)));
+    const F2 P = fma_(dup(C.xi), log1p01<PairArith>(ex), pk(fmaxf(D0, 0.0f), fmaxf(D1, 0.0f)));
     const F2 Pp = pk(D0 >= 0.0f ? lo(inv) : lo(exi), D1 >= 0.0f ? hi(inv) : hi(exi));
     const F2 rs = pk(rsqrtf(fmaxf(lo(P), 1e-37f)), rsqrtf(fmaxf(hi(P), 1e-37f)));
     r = P * rs;
@@ -202,7 +194,7 @@ __device__ __forceinline__ F2 pair_eval(const Coef2& C, F2 u0, F2 dx, F2 dy, F2 
     }
     if constexpr (!GRAD) return e;
     const F2 k = a3 * rp;                                     // de/dD
-    const F2 dT = fma_(C.c2x2, Tr, fma_(C.c3, r, fma_(C.c4, q, (Tr * mtwo) * k)));
+    const F2 dT = fma_(C.c2, Tr + Tr, fma_(C.c3, r, fma_(C.c4, q, (Tr * mtwo) * k)));
     const F2 dq = fma_(C.c4, Tr, C.c5 * r);
     const F2 s2 = two * fma_(two, k, C.c1);
     // Lambda = de/dM = 2 dS M + dT I

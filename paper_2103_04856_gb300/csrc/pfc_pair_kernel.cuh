@@ -81,7 +81,6 @@ __device__ __forceinline__ void field_coefs(const float* c, int plane, Coef2& C)
     F2* const to[NCF] = { &C.c1, &C.c2, &C.c3, &C.c4, &C.c5, &C.c6 };
 #pragma unroll
     for (int q = 0; q < NCF; ++q) *to[q] = pk(c[q * plane], c[q * plane + CP]);
-    C.c2x2 = C.c2 + C.c2;
     C.c6x2 = C.c6 + C.c6;
 }
 
