@@ -321,8 +321,7 @@ __global__ void __launch_bounds__(PairTile<TY>::NT, 1) k_pair(const __grid_const
                 const F2 g = SYM ? fma_(dup(0.5f), xm - xp, g5) : (g5 + xm) - xp;
                 const float g0 = in0 ? lo(g) : 0.0f, g1 = in1 ? hi(g) : 0.0f;
                 sg = sg + pk(g0, g1);
-                sag += fabsf(g0);
-                sag += fabsf(g1);
+                sag += fabsf(g0) + fabsf(g1);   // a term per plane: a term per row rounds twice as often
                 gmax = fmaxf(gmax, fabsf(g0));
                 gmax = fmaxf(gmax, fabsf(g1));
                 if (MODE == MODE_GRAD) {
