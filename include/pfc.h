@@ -70,8 +70,14 @@ typedef struct {
     double eps;             /* interface width > 0 (eq. Meps)                            */
     double xi;              /* regularisation > 0 (Sec. 4.1; 1e-6 in the paper)          */
     double a[6];            /* a20 a11 a02 a10 a01 a00 of eq. F, kappa1 >= kappa2         */
-    int32_t tile_y;         /* tile height: 0 = automatic (FP64: 8; FP32: 16); else 8, 13 or 16.  FP32 tiles
-                               hold an even number of rows: 16 selects 20, 13 selects 12 */
+    /* Tile height: 0 = automatic, else 8, 13 or 16.  FP32: a hint for gradients
+     * and steps of small launches (at most four planes of 20-row tiles per SM),
+     * where 8 selects 8 rows and 13 selects 12; every other FP32 launch, and 16,
+     * takes the automatic height (20 rows, or 28 for symmetric polynomials where
+     * that pads less; 24 or 30 for the energy alone).  FP64: the fused sweep with
+     * that many rows; a nonzero tile_y or tile_z also keeps grids of up to 2^22
+     * voxels off the two-kernel form that is automatic there and faster. */
+    int32_t tile_y;
     int32_t tile_z;         /* 0 = automatic; else planes per CTA z-chunk (>= 1)         */
     /* Orientation term of Sec. 5.2: eps mu (theta . grad u)^2 joins the
      * integrand (grad u the central-difference gradient).  mu = 0 (with any

@@ -134,10 +134,6 @@ template <typename T>
 Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, double mu = 0.0,
                   const double* theta = nullptr, int proj = 0, int refine = 1);
 
-// Tile rows of the packed FP32 sweep (k_pair) for a height hint
-// (pfc_problem.tile_y): its tiles hold an even number of rows.
-inline int pair_tile_rows(int tile_y) { return tile_y == 8 ? 8 : tile_y == 13 ? 12 : 20; }
-
 // Automatic tile height (as a hint): FP64 8 rows, FP32 the tallest.
 inline int default_tile_y(int ny, bool fp64)
 {

@@ -617,6 +617,18 @@ static inline int plane_cost(int rows, bool energy)
     return 16 + (energy ? r : r + 2 - rows % 2);
 }
 
+// work units of the launch's problems in tiles of TY rows
+template <int MAXI>
+static long long pair_units(const Launch<float, MAXI>& L, int TY)
+{
+    long long units = 0;
+    for (int k = 0; k < L.n; ++k) {
+        const Inst<float>& in = L.inst[k];
+        units += (long long)((in.nx + TX - 1) / TX) * ((in.ny + TY - 1) / TY) * in.nz;
+    }
+    return units;
+}
+
 template <int MAXI>
 static void plan_pair(Launch<float, MAXI>& L, int TY, bool energy, int max_run)
 {
@@ -711,14 +723,27 @@ static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStre
     return cudaGetLastError();
 }
 
-// tile_y: the height hint (pfc_problem.tile_y: 8, 13 or 16)
+// Tile rows for the height hint tile_y (pfc_problem.tile_y: 8, 13 or 16): 8 or
+// 12 while there are at most four planes of 20 rows per SM, where the smaller
+// tiles' shorter shares can pay (a 48^3 gradient 17.2 us in 20 rows, 14.7 in
+// 12; 64^3 17.1, 17.5 and, in 8, 18.9).  With more planes they never did
+// (100^3: 28.6, 31.3, 37.6 us; a symmetric 512^3: 958, 1277, 1680 us, where the
+// one-voxel sweep's tiles of 13 and 8 rows had taken 1162 and 1364), so the
+// hint is not followed there.
+template <int MAXI>
+static int pair_rows(const Launch<float, MAXI>& L, int tile_y)
+{
+    const int rows = tile_y == 8 ? 8 : tile_y == 13 ? 12 : 20;
+    return pair_units(L, 20) > 4LL * device_sms() ? 20 : rows;
+}
+
 template <int MAXI, bool SYM, bool HALO>
 static cudaError_t launch_pair_mode(Launch<float, MAXI>& L, int mode, int tile_y, int max_run, cudaStream_t s)
 {
     if constexpr (MAXI == 1) {
         if (mode == MODE_ENERGY) return launch_pair_energy<SYM, HALO>(L, max_run, s);
     }
-    const int rows = pair_tile_rows(tile_y);
+    const int rows = pair_rows(L, tile_y);
     if constexpr (SYM) {
         if (rows == 20 && sym_tall(L))
             return mode == MODE_GRAD   ? launch_pair_one<28, MODE_GRAD, MAXI, SYM, HALO>(L, max_run, s)
