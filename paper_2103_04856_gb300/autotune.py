@@ -1,15 +1,17 @@
 """Launch-shape autotuner for the fused sweep.
 
-The sweep's tile height (32 x 8 or 32 x 16 columns per CTA) and the cap on
-planes a CTA processes per problem (0 = one CTA per SM with equal shares)
-trade halo recomputation, registers and balance against each other, and the
-best choice depends on the grid sizes.  `tune` times every candidate with
+The sweep's tile height (``tile_y``, a hint that launches of few planes per SM
+follow: 32 x 8, 12 or 20 columns per CTA) and the cap on planes a CTA
+processes per problem (0 = one CTA per SM with equal shares) trade halo
+recomputation, registers and balance against each other, and the best choice
+depends on the grid sizes.  `tune` times every candidate with
 CUDA events on synthetic noise fields of the requested shapes (L2 flushed
 between steps, medians of repeated steps) through the library's own batched
 step, and caches the winner in a JSON file keyed by GPU name, precision, the
-multiset of shapes and whether the polynomials are symmetric in kappa1,
-kappa2 (those problems run another instantiation of the sweep, without the
-sqrt(D+) terms, whose best tile can differ).
+sweep that was timed (``SWEEP``: a winner of another sweep's tiles says nothing
+of this one's), the multiset of shapes and whether the polynomials are
+symmetric in kappa1, kappa2 (those problems run another instantiation of the
+sweep, without the sqrt(D+) terms, whose best tile can differ).
 
     from paper_2103_04856_gb300 import autotune
     best = autotune.tune([(128, 128, 128)] * 4)        # {'tile_y': 16, 'max_run': 0, ...}
@@ -35,13 +37,14 @@ CANDIDATES = [
     {"tile_y": 16, "max_run": 32},
     {"tile_y": 8, "max_run": 64},
 ]
+SWEEP = "pair20"      # changes with the sweep's tiles
 DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "autotune_cache.json")
 
 
 def cache_key(shapes, prec: str = "fp32", symmetric: bool = False) -> str:
     dev = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
     shp = ",".join("x".join(str(int(d)) for d in s) for s in sorted(tuple(s) for s in shapes))
-    return f"{dev}|{prec}|{shp}" + ("|sym" if symmetric else "")
+    return f"{dev}|{prec}|{SWEEP}|{shp}" + ("|sym" if symmetric else "")
 
 
 def _load(path):
