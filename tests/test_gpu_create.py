@@ -1,0 +1,74 @@
+"""Contexts are cheap to make and close, and any number of them returns its energies: more than share a
+page of mapped words, and several threads that make, use and close theirs at once."""
+import threading
+import time
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytestmark = [pytest.mark.gpu, pytest.mark.skip(reason="needs a GPU")]
+else:
+    pytestmark = pytest.mark.gpu
+
+from paper_2103_04856_gb300 import inputs as I  # noqa: E402
+from paper_2103_04856_gb300 import pfc  # noqa: E402
+
+A = (0.8, 0.3, 1.1, 0.4, -0.2, 0.1)
+SHAPE = (6, 10, 12)
+
+
+def _prob(shape=SHAPE):
+    return pfc.Problem.from_shape(shape, eps=1.5, a=A, xi=1e-2)
+
+
+def test_making_and_closing_a_context():
+    """Allocating and freeing one word of mapped host memory takes 280 us or more here; a context of the
+    size made 44 us without one."""
+    took = []
+    for _ in range(60):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        pfc.Context(_prob((32, 32, 32))).close()
+        took.append(time.perf_counter() - t)
+    assert np.median(took[10:]) < 200e-6
+
+
+def test_more_contexts_than_words():
+    us = [torch.tensor(I.noise(SHAPE, 0.3, 0.1, k), dtype=torch.float32, device="cuda") for k in range(3)]
+    one = pfc.Context(_prob())
+    want = [one.energy(u) for u in us]
+    ctxs = [pfc.Context(_prob()) for _ in range(600)]
+    for k, c in enumerate(ctxs):
+        assert c.energy(us[k % 3]) == want[k % 3]
+        assert c.energy_and_grad(us[(k + 1) % 3])[0] == pytest.approx(want[(k + 1) % 3], rel=1e-6)
+    for c in ctxs:
+        c.close()
+    again = pfc.Context(_prob())
+    assert again.energy(us[0]) == want[0] and one.energy(us[1]) == want[1]
+
+
+def test_threads_make_use_and_close_contexts():
+    us = [torch.tensor(I.noise(SHAPE, 0.3, 0.1, k), dtype=torch.float32, device="cuda") for k in range(4)]
+    one = pfc.Context(_prob())
+    want = [one.energy(u) for u in us]
+    errors = []
+
+    def job(k):
+        try:
+            s = torch.cuda.Stream()
+            for _ in range(25):
+                c = pfc.Context(_prob())
+                for _ in range(3):
+                    assert c.energy(us[k], stream=s) == want[k]
+                c.close()
+        except Exception as e:          # reported after the join
+            errors.append(e)
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=job, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
