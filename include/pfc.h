@@ -110,7 +110,10 @@ typedef struct pfc_ctx pfc_ctx;
 
 /* Validates the problem and allocates the context's device scratch
  * (ping-pong field, FP64 block partials, scalars; the plain path adds 21
- * fields).  The current CUDA device at this call is the context's device. */
+ * fields; FP64 problems that take the two-kernel form, see tile_y, add 10
+ * fields of doubles, 80 bytes a voxel, also where a coefficient field is set
+ * later; without that much memory they run the fused sweep).  The current CUDA
+ * device at this call is the context's device. */
 pfc_status pfc_create(const pfc_problem* prob, pfc_ctx** out);
 void pfc_destroy(pfc_ctx* ctx);
 
@@ -212,7 +215,9 @@ enum { PFC_SLAB_ENERGY = 0, PFC_SLAB_GRAD = 1, PFC_SLAB_STEP = 2 };
 /* prob: the WHOLE grid (nx, ny, nz global), fused path, FP32 or FP64 (mu and
  * proj allowed; no coefficient field).  This slab holds planes
  * [z0, z0 + nz_local), nz_local >= 2, inside [0, nz).  Allocates the slab's
- * FP64 partials and scalars (not its fields). */
+ * FP64 partials and scalars (not its fields), and for FP64 slabs of up to 2^22
+ * voxels the two-kernel form's 80 bytes a voxel of nz_local + 2 planes (without
+ * that much memory the slab runs the fused sweep). */
 pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32_t nz_local, pfc_slab** out);
 void pfc_slab_destroy(pfc_slab* slab);
 /* One sweep over the slab.  u: the slab's nz_local planes (device, layout of

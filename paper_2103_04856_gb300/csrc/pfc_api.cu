@@ -13,6 +13,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/pfc.h"
+#include "pfc_alloc.h"
 #include "pfc_internal.h"
 #include "pfc_words.h"
 
@@ -53,8 +54,9 @@ void set_last_error(const char* msg) { snprintf(g_err, sizeof g_err, "%s", msg);
 // ------------------------------------------------------------ context
 
 // Mapped host memory for the energies that calls wait for: 4 KB per device for
-// all contexts.  Allocating and freeing a word for each made creating and
-// closing a 32^3 context 362 us instead of 44.
+// all contexts.  A word of its own made creating and closing a 32^3 context
+// 490 us instead of 192 (362 instead of 44 beside a context that keeps the
+// allocator's block of small memory mapped).
 struct EnergyPage {
     static double* make()
     {
@@ -90,7 +92,7 @@ struct pfc_ctx {
     double* trace = nullptr;
     int trace_cap = 0;
     void* plain_mem = nullptr;       // 21 fields for the plain path
-    void* work = nullptr;            // small FP64 grids: cotangents (launch_split)
+    void* work = nullptr;            // small FP64 grids: cotangents (launch_split), in ping's block; or null: the sweep
     void* cfield = nullptr;          // c(x) from pfc_set_coefficient_field (NCF fields)
     bool cf_on = false;
     double* dpart = nullptr;         // diagnostics: block partials, ticket, 5 results
@@ -201,6 +203,14 @@ static size_t split_bytes(const pfc_problem* p, int nz, int extra)
     return split_work((long)p->nx * p->ny * (nz + extra));
 }
 
+static void* device_alloc(size_t bytes)
+{
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    (void)cudaGetLastError();
+    return nullptr;
+}
+
 static void free_ctx_mem(pfc_ctx* c)
 {
     cudaFree(c->ping);
@@ -211,7 +221,6 @@ static void free_ctx_mem(pfc_ctx* c)
     cudaFree(c->trace);
     cudaFree(c->plain_mem);
     cudaFree(c->cfield);
-    cudaFree(c->work);
     cudaFree(c->dpart);
     cudaFree(c->dticket);
     cudaFree(c->dout);
@@ -244,16 +253,16 @@ extern "C" pfc_status pfc_create(const pfc_problem* prob, pfc_ctx** out)
     c->nblocks = (int)fused_grid(fused_units(prob->nx, prob->ny, prob->nz), prob->tile_z);
     c->plain_nblocks = plain_blocks(c->N);
     const int nparts = c->nblocks > c->plain_nblocks ? c->nblocks : c->plain_nblocks;
-    bool ok = cudaMalloc(&c->ping, (size_t)c->esz * c->N) == cudaSuccess &&
-              cudaMalloc((void**)&c->partials, sizeof(double) * NPART * (size_t)nparts) == cudaSuccess &&
+    const bool fused = prob->impl == PFC_IMPL_FUSED;
+    bool ok = cudaMalloc((void**)&c->partials, sizeof(double) * NPART * (size_t)nparts) == cudaSuccess &&
               cudaMalloc((void**)&c->ints, sizeof(unsigned) * NINTS) == cudaSuccess &&
               cudaMalloc((void**)&c->scal, sizeof(double) * NSCAL) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess;
-    if (ok && prob->impl == PFC_IMPL_FUSED) {
+              cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) == cudaSuccess &&
+              alloc_with_work(device_alloc, (size_t)c->esz * c->N, fused ? split_bytes(prob, prob->nz, 0) : 0, &c->ping,
+                              &c->work);
+    if (ok && fused) {
         if (c->device < 64) c->e_word = g_energy_words[c->device].take();
         c->e_host = c->e_word.p;
-        const size_t bytes = split_bytes(prob, prob->nz, 0);
-        if (ok && bytes) ok = cudaMalloc(&c->work, bytes) == cudaSuccess;
     }
     if (ok && prob->impl == PFC_IMPL_PLAIN)
         ok = cudaMalloc(&c->plain_mem, (size_t)c->esz * c->N * 21) == cudaSuccess;
@@ -265,7 +274,8 @@ extern "C" pfc_status pfc_create(const pfc_problem* prob, pfc_ctx** out)
         cudaError_t le = cudaGetLastError();
         free_ctx_mem(c);
         delete c;
-        return fail(PFC_ENOMEM, "device allocation failed: %s", cudaGetErrorString(le));
+        return fail(PFC_ENOMEM, "device allocation failed: %s",
+                    cudaGetErrorString(le == cudaSuccess ? cudaErrorMemoryAllocation : le));
     }
     *out = c;
     return PFC_OK;
@@ -726,7 +736,7 @@ struct pfc_slab {
     double* partials = nullptr;
     double* scal = nullptr;
     unsigned* ints = nullptr;
-    void* work = nullptr;   // small FP64 slabs: cotangents (launch_split)
+    void* work = nullptr;   // small FP64 slabs: cotangents (launch_split), in mem's block; or null: the sweep
     int last_mode = -1;     // mode of the last sweep: what pfc_slab_finish combines
 };
 
@@ -757,10 +767,7 @@ extern "C" pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32
     sl->nblocks = (int)fused_grid(fused_units(prob->nx, prob->ny, nz_local), prob->tile_z);
     const size_t bytes = sizeof(double) * ((size_t)NPART * sl->nblocks + NSCAL) + sizeof(unsigned) * NINTS;
     const size_t wbytes = split_bytes(prob, nz_local, 2);
-    if (cudaMalloc((void**)&sl->mem, bytes) != cudaSuccess ||
-        (wbytes && cudaMalloc(&sl->work, wbytes) != cudaSuccess)) {
-        (void)cudaGetLastError();
-        cudaFree(sl->mem);
+    if (!alloc_with_work(device_alloc, bytes, wbytes, (void**)&sl->mem, &sl->work)) {
         delete sl;
         return fail(PFC_ENOMEM, "device allocation of %zu bytes failed", bytes);
     }
@@ -774,7 +781,6 @@ extern "C" pfc_status pfc_slab_create(const pfc_problem* prob, int32_t z0, int32
         cudaError_t e = cudaGetLastError();
         if (s) cudaStreamDestroy(s);
         cudaFree(sl->mem);
-        cudaFree(sl->work);
         delete sl;
         return fail(PFC_ECUDA, "clearing the slab's scalars failed: %s", cudaGetErrorString(e));
     }
@@ -791,7 +797,6 @@ extern "C" void pfc_slab_destroy(pfc_slab* sl)
     cudaSetDevice(sl->device);
     cudaDeviceSynchronize();
     cudaFree(sl->mem);
-    cudaFree(sl->work);
     cudaSetDevice(prev);
     delete sl;
 }
