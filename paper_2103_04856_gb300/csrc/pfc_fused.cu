@@ -77,10 +77,54 @@ cudaError_t launch_slab_finish(const double* rows, int nslabs, double inv_N, int
     return cudaGetLastError();
 }
 
-// Diffuse principal curvatures (Sec. 3.1, eqs. kepsa/kepsb) per voxel.  A
-// block of 32 x 8 columns marches up a chunk of zc planes; a thread keeps the
-// 3 x 3 neighbourhood of its column on the planes z - 1, z, z + 1 in registers
-// and loads that of the next plane (9 loads a voxel, from L1 but for its own).
+// Diffuse principal curvatures (Sec. 3.1, eqs. kepsa/kepsb) of a voxel;
+// at(dx, dy, dz): u at that offset.
+template <typename T, class At>
+__device__ __forceinline__ void voxel_curvatures(const At& at, const Coef<T>& C, T eps, T* k1, T* k2)
+{
+    const T u0 = at(0, 0, 0);
+    const T dx = at(1, 0, 0) - at(-1, 0, 0), dy = at(0, 1, 0) - at(0, -1, 0), dz = at(0, 0, 1) - at(0, 0, -1);
+    const T hxx = at(1, 0, 0) + at(-1, 0, 0) - T(2) * u0;
+    const T hyy = at(0, 1, 0) + at(0, -1, 0) - T(2) * u0;
+    const T hzz = at(0, 0, 1) + at(0, 0, -1) - T(2) * u0;
+    const T hxy = at(1, 1, 0) - at(1, -1, 0) - at(-1, 1, 0) + at(-1, -1, 0);
+    const T hxz = at(1, 0, 1) - at(1, 0, -1) - at(-1, 0, 1) + at(-1, 0, -1);
+    const T hyz = at(0, 1, 1) - at(0, 1, -1) - at(0, -1, 1) + at(0, -1, -1);
+    const T Gx = dx * C.sg, Gy = dy * C.sg, Gz = dz * C.sg;
+    const T rho = Gx * Gx + Gy * Gy + Gz * Gz + C.xi2;
+    T Mxx, Myy, Mzz, Mxy, Mxz, Myz;
+    if (C.proj) {   // M = P K P, K = -eps Hess u, P = I - G G^T / rho
+        const T Kxx = C.kd * hxx, Kyy = C.kd * hyy, Kzz = C.kd * hzz;
+        const T Kxy = C.ko * hxy, Kxz = C.ko * hxz, Kyz = C.ko * hyz;
+        const T kx = Kxx * Gx + Kxy * Gy + Kxz * Gz, ky = Kxy * Gx + Kyy * Gy + Kyz * Gz;
+        const T kz = Kxz * Gx + Kyz * Gy + Kzz * Gz;
+        const T s = Gx * kx + Gy * ky + Gz * kz;
+        const T ir = T(1) / rho, s2 = s * ir * ir;
+        Mxx = Kxx - T(2) * ir * Gx * kx + s2 * Gx * Gx;
+        Myy = Kyy - T(2) * ir * Gy * ky + s2 * Gy * Gy;
+        Mzz = Kzz - T(2) * ir * Gz * kz + s2 * Gz * Gz;
+        Mxy = Kxy - ir * (Gx * ky + kx * Gy) + s2 * Gx * Gy;
+        Mxz = Kxz - ir * (Gx * kz + kx * Gz) + s2 * Gx * Gz;
+        Myz = Kyz - ir * (Gy * kz + ky * Gz) + s2 * Gy * Gz;
+    } else {
+        const T wp = C.well == 0 ? T(2) * u0 * (T(1) - u0) * (T(1) - T(2) * u0) : u0 * u0 * u0 - u0;
+        const T wr = wp * C.inv_eps / rho;
+        Mxx = C.kd * hxx + wr * Gx * Gx; Myy = C.kd * hyy + wr * Gy * Gy; Mzz = C.kd * hzz + wr * Gz * Gz;
+        Mxy = C.ko * hxy + wr * Gx * Gy; Mxz = C.ko * hxz + wr * Gx * Gz; Myz = C.ko * hyz + wr * Gy * Gz;
+    }
+    const T Tr = Mxx + Myy + Mzz;
+    const T S = Mxx * Mxx + Myy * Myy + Mzz * Mzz + T(2) * (Mxy * Mxy + Mxz * Mxz + Myz * Myz);
+    const T D = T(2) * S - Tr * Tr;
+    const T root = sqrt_(D > T(0) ? D : T(0));
+    const T den = T(2) * eps * sqrt_(rho);
+    *k1 = (Tr + root) / den;
+    *k2 = (Tr - root) / den;
+}
+
+// FP32: a block of 32 x 8 columns marches up a chunk of zc planes; a thread
+// keeps the 3 x 3 neighbourhood of its column on the planes z - 1, z, z + 1 in
+// registers and loads that of the next plane (9 loads a voxel, from L1 but for
+// its own).
 // 4 B read and 8 B written a voxel; a voxel at a time in a grid-stride loop,
 // with two 64-bit divisions and 19 wrapped neighbours, it took 148 us at 200^3
 // (0.65 TB/s); now 71 us, bound by instruction issue (240 a voxel, a quarter of
@@ -123,47 +167,29 @@ __global__ void __launch_bounds__(kCurvX* kCurvY) k_curvatures(const T* __restri
             const int j = 3 * (ddy + 1) + ddx + 1;
             return ddz < 0 ? a[j] : ddz > 0 ? c[j] : b[j];
         };
-        const T u0 = at(0, 0, 0);
-        const T dx = at(1, 0, 0) - at(-1, 0, 0), dy = at(0, 1, 0) - at(0, -1, 0), dz = at(0, 0, 1) - at(0, 0, -1);
-        const T hxx = at(1, 0, 0) + at(-1, 0, 0) - T(2) * u0;
-        const T hyy = at(0, 1, 0) + at(0, -1, 0) - T(2) * u0;
-        const T hzz = at(0, 0, 1) + at(0, 0, -1) - T(2) * u0;
-        const T hxy = at(1, 1, 0) - at(1, -1, 0) - at(-1, 1, 0) + at(-1, -1, 0);
-        const T hxz = at(1, 0, 1) - at(1, 0, -1) - at(-1, 0, 1) + at(-1, 0, -1);
-        const T hyz = at(0, 1, 1) - at(0, 1, -1) - at(0, -1, 1) + at(0, -1, -1);
-        const T Gx = dx * C.sg, Gy = dy * C.sg, Gz = dz * C.sg;
-        const T rho = Gx * Gx + Gy * Gy + Gz * Gz + C.xi2;
-        T Mxx, Myy, Mzz, Mxy, Mxz, Myz;
-        if (C.proj) {   // M = P K P, K = -eps Hess u, P = I - G G^T / rho
-            const T Kxx = C.kd * hxx, Kyy = C.kd * hyy, Kzz = C.kd * hzz;
-            const T Kxy = C.ko * hxy, Kxz = C.ko * hxz, Kyz = C.ko * hyz;
-            const T kx = Kxx * Gx + Kxy * Gy + Kxz * Gz, ky = Kxy * Gx + Kyy * Gy + Kyz * Gz;
-            const T kz = Kxz * Gx + Kyz * Gy + Kzz * Gz;
-            const T s = Gx * kx + Gy * ky + Gz * kz;
-            const T ir = T(1) / rho, s2 = s * ir * ir;
-            Mxx = Kxx - T(2) * ir * Gx * kx + s2 * Gx * Gx;
-            Myy = Kyy - T(2) * ir * Gy * ky + s2 * Gy * Gy;
-            Mzz = Kzz - T(2) * ir * Gz * kz + s2 * Gz * Gz;
-            Mxy = Kxy - ir * (Gx * ky + kx * Gy) + s2 * Gx * Gy;
-            Mxz = Kxz - ir * (Gx * kz + kx * Gz) + s2 * Gx * Gz;
-            Myz = Kyz - ir * (Gy * kz + ky * Gz) + s2 * Gy * Gz;
-        } else {
-            const T wp = C.well == 0 ? T(2) * u0 * (T(1) - u0) * (T(1) - T(2) * u0) : u0 * u0 * u0 - u0;
-            const T wr = wp * C.inv_eps / rho;
-            Mxx = C.kd * hxx + wr * Gx * Gx; Myy = C.kd * hyy + wr * Gy * Gy; Mzz = C.kd * hzz + wr * Gz * Gz;
-            Mxy = C.ko * hxy + wr * Gx * Gy; Mxz = C.ko * hxz + wr * Gx * Gz; Myz = C.ko * hyz + wr * Gy * Gz;
-        }
-        const T Tr = Mxx + Myy + Mzz;
-        const T S = Mxx * Mxx + Myy * Myy + Mzz * Mzz + T(2) * (Mxy * Mxy + Mxz * Mxz + Myz * Myz);
-        const T D = T(2) * S - Tr * Tr;
-        const T root = sqrt_(D > T(0) ? D : T(0));
-        const T den = T(2) * eps * sqrt_(rho);
-        *o1 = (Tr + root) / den;
-        *o2 = (Tr - root) / den;
+        voxel_curvatures<T>(at, C, eps, o1, o2);
         o1 += pls;
         o2 += pls;
 #pragma unroll
         for (int j = 0; j < 9; ++j) { a[j] = b[j]; b[j] = c[j]; }
+    }
+}
+
+// FP64: a voxel at a time.  Bound by the FP64 roots and quotients, so what
+// counts is that every lane has a voxel and the last wave is full; the march's
+// padded rows, longer blocks and chunks of eight planes made 200^3 1.54 -> 1.90
+// ms, 100^3 0.20 -> 0.31 ms and 16^3 18 -> 69 us.
+__global__ void __launch_bounds__(256) k_curvatures_each(const double* __restrict__ u, double* __restrict__ k1,
+                                                         double* __restrict__ k2, int nx, int ny, int nz,
+                                                         Coef<double> C, double eps)
+{
+    const long n = (long)nx * ny * nz;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((long)nx * ny));
+        auto at = [&](int dx, int dy, int dz) {
+            return __ldg(u + ((long)wrapi(z + dz, nz) * ny + wrapi(y + dy, ny)) * nx + wrapi(x + dx, nx));
+        };
+        voxel_curvatures<double>(at, C, eps, k1 + i, k2 + i);
     }
 }
 
@@ -401,14 +427,19 @@ template <typename T>
 cudaError_t launch_curvatures(const T* u, T* k1, T* k2, int nx, int ny, int nz, const Coef<T>& C, double eps,
                               cudaStream_t s)
 {
-    const long tiles_x = (nx + kCurvX - 1) / kCurvX, tiles = tiles_x * ((ny + kCurvY - 1) / kCurvY);
-    // chunks of planes so that about 16 blocks per SM share the work, no shorter than 8 planes
-    // (a chunk loads two planes more than it writes)
-    int zc = nz;
-    while (zc > 8 && tiles * ((nz + zc - 1) / zc) < 16L * device_sms()) zc = (zc + 1) / 2;
-    const int chunks = (nz + zc - 1) / zc;
-    k_curvatures<T><<<(unsigned)(tiles * chunks), dim3(kCurvX, kCurvY), 0, s>>>(u, k1, k2, nx, ny, nz, (int)tiles_x,
-                                                                               chunks, zc, C, (T)eps);
+    if constexpr (sizeof(T) == 8) {
+        const long n = (long)nx * ny * nz, b = (n + 255) / 256, most = 16L * device_sms();
+        k_curvatures_each<<<(unsigned)(b < most ? b : most), 256, 0, s>>>(u, k1, k2, nx, ny, nz, C, eps);
+    } else {
+        const long tiles_x = (nx + kCurvX - 1) / kCurvX, tiles = tiles_x * ((ny + kCurvY - 1) / kCurvY);
+        // chunks of planes so that about 16 blocks per SM share the work, no shorter than 8 planes
+        // (a chunk loads two planes more than it writes)
+        int zc = nz;
+        while (zc > 8 && tiles * ((nz + zc - 1) / zc) < 16L * device_sms()) zc = (zc + 1) / 2;
+        const int chunks = (nz + zc - 1) / zc;
+        k_curvatures<T><<<(unsigned)(tiles * chunks), dim3(kCurvX, kCurvY), 0, s>>>(u, k1, k2, nx, ny, nz, (int)tiles_x,
+                                                                                   chunks, zc, C, (T)eps);
+    }
     return cudaGetLastError();
 }
 template cudaError_t launch_curvatures<float>(const float*, float*, float*, int, int, int, const Coef<float>&,
