@@ -31,6 +31,7 @@
 #include <type_traits>
 
 #include "pfc_device.cuh"
+#include "pfc_once.h"
 
 namespace pfc {
 
@@ -400,19 +401,27 @@ k_fused(const __grid_constant__ Launch<T, 1> L)
 
 size_t fused_smem_bytes(int elem_size, int tile_y);
 
-// One launch of k_fused (sets the dynamic shared-memory limit once per
-// instantiation; idempotent, so a race between threads is harmless).
+// Allows `kernel` more than 48 KB of dynamic shared memory on the current
+// device (the attribute is the device's own).
+template <typename Kernel>
+static cudaError_t allow_smem(OncePerDevice& once, Kernel kernel, size_t smem)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once(dev, [&] {
+        return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
+}
+
+// One launch of k_fused.
 template <typename T, int TY, int MODE, int EXT = 0, bool HALO = false>
 static cudaError_t launch_kernel(const Launch<T, 1>& L, int blocks, cudaStream_t s)
 {
     const size_t smem = fused_smem_bytes(sizeof(T), TY);
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k_fused<T, TY, MODE, EXT, HALO>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, k_fused<T, TY, MODE, EXT, HALO>, smem);
+    if (e != cudaSuccess) return e;
     k_fused<T, TY, MODE, EXT, HALO><<<blocks, Tile<TY>::NT, smem, s>>>(L);
     return cudaGetLastError();
 }

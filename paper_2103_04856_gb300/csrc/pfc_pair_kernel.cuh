@@ -695,13 +695,9 @@ static cudaError_t launch_pair_one(Launch<float, MAXI>& L, int max_run, cudaStre
 {
     plan_pair(L, TY, false, max_run);
     const size_t smem = PairTile<TY>::SMEM + (EXT == 2 ? PairTile<TY>::CSMEM : 0);
-    static bool attr_done = false;   // idempotent, so a race between threads is harmless
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k_pair<TY, MODE, MAXI, SYM, HALO, EXT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, k_pair<TY, MODE, MAXI, SYM, HALO, EXT>, smem);
+    if (e != cudaSuccess) return e;
     k_pair<TY, MODE, MAXI, SYM, HALO, EXT><<<L.grid, PairTile<TY>::NT, smem, s>>>(L);
     return cudaGetLastError();
 }
@@ -712,13 +708,9 @@ static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStre
     using TL = PairEnergyTile<SYM>;
     plan_pair(L, TL::TY, true, max_run);
     const size_t smem = TL::SMEM + (EXT == 2 ? TL::CSMEM : 0);
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k_pair_energy<SYM, HALO, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, k_pair_energy<SYM, HALO, EXT>, smem);
+    if (e != cudaSuccess) return e;
     k_pair_energy<SYM, HALO, EXT><<<L.grid, TL::NT, smem, s>>>(L);
     return cudaGetLastError();
 }
