@@ -22,8 +22,10 @@
  *  - Fields are caller-owned device arrays u[(z*ny + y)*nx + x] (torch shape
  *    (nz, ny, nx), contiguous), of float (PFC_FP32) or double (PFC_FP64) as the
  *    problem says, on the current CUDA device.  The library never frees them.
- *    A base address that is not 16-byte aligned, or nx not a multiple of
- *    16/sizeof(element), selects a slower element-wise load path (not an error).
+ *    Any base address and any nx will do; where they are not multiples of 16
+ *    bytes, the FP64 sweep, the sweep of the projected M, coefficient fields,
+ *    the diagnostics, the surface cells and Alg. 1's passes load element by
+ *    element, which is slower (the plain FP32 sweep does not).
  *  - The stream is a cudaStream_t (NULL = the legacy default stream).  Work is
  *    enqueued on it in order; entry points with a host output wait for it.
  *  - Errors are returned as pfc_status; pfc_last_error() gives a message for

@@ -146,7 +146,7 @@ static pfc_status check_problem(const pfc_problem* p)
 // so that the grid fills the GPU about twice unless the user fixed tile_z.
 static void geometry(const pfc_problem* p, int sms, int* tile_y, int* zc, int* tx, int* ty, int* cz)
 {
-    int tyv = p->tile_y ? p->tile_y : default_tile_y(p->ny, p->prec == PFC_FP64);
+    int tyv = p->tile_y ? p->tile_y : default_tile_y(p->prec == PFC_FP64);
     *tile_y = tyv;
     *tx = (p->nx + 31) / 32;
     *ty = (p->ny + tyv - 1) / tyv;
@@ -955,7 +955,7 @@ extern "C" pfc_status pfc_batch_create(const pfc_problem* probs, int32_t n, pfc_
     b->host.resize(n);
     b->ping.assign(n, nullptr);
     bool ok = true;
-    b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(probs[0].ny, false);   // one height for all instances
+    b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(false);   // one height for all instances
     b->max_run = probs[0].tile_z;
     long long units = 0;
     for (int k = 0; k < n && ok; ++k) {

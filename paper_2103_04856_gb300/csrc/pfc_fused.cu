@@ -201,7 +201,7 @@ Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, 
 {
     const double h3 = h * h * h;
     Coef<T> C;
-    memset(&C, 0, sizeof C);   // padding too: batched launches compare coefficient sets bytewise
+    memset(&C, 0, sizeof C);
     C.c1 = (T)((a[0] + a[2] - a[1]) / (2.0 * eps) * h3);
     C.c2 = (T)(a[1] / (2.0 * eps) * h3);
     C.c3 = (T)((a[0] - a[2]) / (2.0 * eps) * h3);
@@ -285,8 +285,6 @@ cudaError_t launch_coef_field(const T* a_field, T* c_field, long n, double h, do
 }
 template cudaError_t launch_coef_field<float>(const float*, float*, long, double, double, cudaStream_t);
 template cudaError_t launch_coef_field<double>(const double*, double*, long, double, double, cudaStream_t);
-
-int fused_threads(int tile_y) { return tile_y == 8 ? Tile<8>::NT : tile_y == 13 ? Tile<13>::NT : Tile<16>::NT; }
 
 size_t fused_smem_bytes(int elem_size, int tile_y)
 {

@@ -21,11 +21,12 @@
 //
 // EXT (the extended sweep): 1 = the orientation term of Sec. 5.2 and
 // coefficients read per voxel from a field c(x) (each thread loads the six
-// coefficients of its column one plane ahead of their use); 2 = the same
-// with the tangent-projected M = -eps P Hess u P.
+// coefficients of its column one plane ahead of their use; FP64); 2 = the same
+// with the tangent-projected M = -eps P Hess u P (FP32 and FP64).
 //
-// FP64 sweeps and the extended ones run here; FP32 without extensions runs two
-// voxels per thread (k_pair, pfc_pair_kernel.cuh).
+// FP64 sweeps (but see pfc_split.cu for small grids) and the projected form run
+// here; all other FP32 sweeps run two voxels per thread (k_pair,
+// pfc_pair_kernel.cuh).
 #pragma once
 
 #include <type_traits>
@@ -105,7 +106,7 @@ template <typename T, int TY, int MODE, int EXT = 0, bool HALO = false>
 __global__ void __launch_bounds__(Tile<TY>::NT, 1)
 k_fused(const __grid_constant__ Launch<T, 1> L)
 {
-    static_assert(EXT != 0 || sizeof(T) == 8, "FP32 without extensions runs k_pair");
+    static_assert(EXT == 2 || sizeof(T) == 8, "FP32 runs k_pair but for the projected form");
     using TL = Tile<TY>;
     constexpr int EX = TL::EX, NEXT = TL::NEXT, NT = TL::NT, UY = TL::UY, PLANE = TL::PLANE;
     constexpr int VEC = 16 / (int)sizeof(T);
@@ -325,16 +326,15 @@ k_fused(const __grid_constant__ Launch<T, 1> L)
                     if constexpr (EXT) return Cv;
                     else return in.C;
                 }();
-                // re-evaluation of D from the exact float inputs (float path only):
-                // double-float for eq. Meps, FP64 for the projected form
+                // re-evaluation of D from the exact float inputs, in FP64 (float only, which
+                // runs the projected form here)
                 auto refine = [&]() -> T {
-                    const T* pm = us + ((m - 1) & (NBUF - 1)) * PLANE + uc;
-                    // (R and the well are the problem's: a coefficient field changes only
-                    // c1 .. c6, and a reference to the per-plane copy Cv would put it in
-                    // local memory)
-                    if constexpr (EXT == 2) return discriminant_fp64_proj_at<T>(in.C.R, pm, p0, pp, UXP);
-                    else if constexpr (EXT == 1) return discriminant_df_at<T>(in.C.R, in.C.well, pm, p0, pp, 1, UXP, -UXP, cind);
-                    else return discriminant_df_at<T>(CC.R, CC.well, pm, p0, pp, 1, UXP, -UXP, cind);
+                    // (R is the problem's: a coefficient field changes only c1 .. c6, and a
+                    // reference to the per-plane copy Cv would put it in local memory)
+                    if constexpr (sizeof(T) == 4)
+                        return discriminant_fp64_proj_at<T>(in.C.R, us + ((m - 1) & (NBUF - 1)) * PLANE + uc, p0, pp, UXP);
+                    else
+                        return T(0);
                 };
                 if constexpr (MODE == MODE_ENERGY) {
                     const T e = voxel_eval<T, false, EXT != 0, EXT == 2>(CC, u0 + cin, dx, dy, dz, hxx, hyy, hzz, hxy, hxz, hyz, ctv, refine);

@@ -965,7 +965,7 @@ extern "C" pfc_status pfc_hflow_create(const pfc_problem* prob, const pfc_hflow_
     h->H.blur_radius = R;
     h->N = (long)p.nx * p.ny * p.nz;
     h->esz = p.prec == PFC_FP64 ? 8 : 4;
-    h->tile_y = p.tile_y ? p.tile_y : default_tile_y(p.ny, p.prec == PFC_FP64);
+    h->tile_y = p.tile_y ? p.tile_y : default_tile_y(p.prec == PFC_FP64);
     h->W.R = R;
     if (R > 0) {   // discrete Gaussian, normalised to sum 1
         double s = 0;
@@ -1450,7 +1450,7 @@ extern "C" pfc_status pfc_hflow_batch_create(const pfc_problem* probs, const dou
             b->W.wf[j + R] = (float)b->W.wd[j + R];
         }
     }
-    b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(b->ny, false);
+    b->tile_y = probs[0].tile_y ? probs[0].tile_y : default_tile_y(false);
     cudaGetDevice(&b->device);
     b->slots = (int)fused_grid(fused_units(b->nx, b->ny, b->nz) * n_inst, probs[0].tile_z);
     b->fblocks = flow_blocks(b->N);

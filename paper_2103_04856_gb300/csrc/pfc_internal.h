@@ -135,11 +135,7 @@ Coef<T> make_coef(const double a[6], double h, double eps, double xi, int well, 
                   const double* theta = nullptr, int proj = 0, int refine = 1);
 
 // Automatic tile height (as a hint): FP64 8 rows, FP32 the tallest.
-inline int default_tile_y(int ny, bool fp64)
-{
-    (void)ny;
-    return fp64 ? 8 : 16;
-}
+inline int default_tile_y(bool fp64) { return fp64 ? 8 : 16; }
 
 // The extended sweep (orientation term, c(x), projected M) runs with 8-row tiles.
 template <typename T>
@@ -169,7 +165,13 @@ long long fused_grid(long long units, int max_run);
 // fused_grid(fused_units(...), max_run).
 long long fused_units(int nx, int ny, int nz);
 // FP64 evaluations without extensions as two kernels, cotangents to memory and
-// the adjoint from it (pfc_split.cu), of problems that bring in.work
+// the adjoint from it (pfc_split.cu), of problems that bring in.work.  Faster
+// than the fused sweep on every grid measured up to SPLIT_MAX (gradients, in us,
+// sweep -> two kernels with a general and a symmetric polynomial: 16^3 75 -> 21 and
+// 17, 64^3 252 -> 155 and 90, 101^3 898 -> 535 and 287, 128^3 1329 -> 1048 and 555,
+// 161^3 3142 -> 1874 and 1081, 1 x 2048 x 2048 6849 -> 1981 and 1085; energies 1.04
+// to 1.5 times and 1.7 to 2.7 times); the line is where the work space, 80 bytes a
+// voxel, reaches a third of a gigabyte.
 constexpr long SPLIT_MAX = 1L << 22;
 // whether a problem (its slab of nz planes) takes them: at most SPLIT_MAX voxels
 bool split_fits(int nx, int ny, int nz, int tile_y, int tile_z, double mu, int proj);
@@ -197,7 +199,6 @@ template <typename T>
 cudaError_t launch_curvatures(const T* u, T* k1, T* k2, int nx, int ny, int nz, const Coef<T>& C,
                               double eps, cudaStream_t s);
 size_t fused_smem_bytes(int elem_size, int tile_y);
-int fused_threads(int tile_y);
 
 // viability diagnostics (pfc_diag.cu): part holds 4 doubles per block
 // (diag_blocks), *ticket starts at 0 and is left at 0, out receives 5 doubles

@@ -102,7 +102,7 @@ static pfc_status run_noalloc(const pfc_problem* p, const void* u, void* g, doub
     in.u = (const T*)u;
     in.out = (T*)g;
     in.nx = p->nx; in.ny = p->ny; in.nz = p->nz;
-    const int tile_y = p->tile_y ? p->tile_y : default_tile_y(p->ny, sizeof(T) == 8);
+    const int tile_y = p->tile_y ? p->tile_y : default_tile_y(sizeof(T) == 8);
     in.tiles_x = (p->nx + 31) / 32;
     in.tiles_y = (p->ny + tile_y - 1) / tile_y;
     in.zc = p->nz;
