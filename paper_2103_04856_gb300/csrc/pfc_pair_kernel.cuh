@@ -534,6 +534,8 @@ __global__ void __launch_bounds__(PairEnergyTile<SYM>::NT, 1) k_pair_energy(cons
             pz = pz + 1 == nz ? 0 : pz + 1;
         };
 #if PFC_DEBUG
+        if constexpr (EXT == 2)
+            for (int i = threadIdx.x; i < CBUF * NCF * TL::CR * CP; i += NT) cs[i] = NAN;
         for (int i = threadIdx.x; i < NBUF * PLANE; i += NT) us[i] = dup(NAN);
         __syncthreads();
 #endif

@@ -5,7 +5,9 @@
 //
 // FP64 runs at 1/64 of the FP32 rate here (two lanes per SM and clock), so a
 // step costs its FP64 operations, not its bytes: about 180 a voxel against 250
-// bytes, which a grid of up to SPLIT_MAX voxels mostly finds in L2.  The fused sweep (k_fused)
+// bytes, which grids of up to 10^6 voxels or so find in L2 (80 bytes a voxel of
+// it at a time); above, they come from HBM, and the operations still take
+// longer.  The fused sweep (k_fused)
 // evaluates the halo of its tiles again, and two planes more per run, which
 // on a 32^3 grid (runs of one plane, 11 warps for 8 rows) is every voxel four
 // times, and always takes the softplus's exp and log1p (about 150 operations),
@@ -264,11 +266,17 @@ static void split(const Inst<double>& in, int mode, cudaStream_t s)
 {
     const long n = (long)in.nx * in.ny * (in.nz + (HALO ? 2 : 0));
     const int nb = split_blocks(n);
+#if PFC_DEBUG
+    cudaMemsetAsync(in.work, 0xff, split_work(n), s);   // NaN
+    const bool chained = false;
+#else
+    const bool chained = in.chained != 0;
+#endif
     if (mode == MODE_ENERGY) {
-        launch_chained(in.chained != 0, k_cot<SYM, false, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
+        launch_chained(chained, k_cot<SYM, false, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
         return;
     }
-    launch_chained(in.chained != 0, k_cot<SYM, true, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
+    launch_chained(chained, k_cot<SYM, true, HALO>, nb, kThreads, 0, s, in, (int)n, mode, in.work);
     if (mode == MODE_GRAD) launch_chained(true, k_adj<SYM, MODE_GRAD, HALO>, nb, kThreads, 0, s, in, (int)n, in.work);
     else launch_chained(true, k_adj<SYM, MODE_STEP, HALO>, nb, kThreads, 0, s, in, (int)n, in.work);
 }
