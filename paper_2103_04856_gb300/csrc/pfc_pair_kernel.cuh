@@ -724,15 +724,17 @@ static cudaError_t launch_pair_energy(Launch<float, 1>& L, int max_run, cudaStre
 // Tile rows for the height hint tile_y (pfc_problem.tile_y: 8, 13 or 16): 8 or
 // 12 while there are at most four planes of 20 rows per SM, where the smaller
 // tiles' shorter shares can pay (a 48^3 gradient 17.2 us in 20 rows, 14.7 in
-// 12; 64^3 17.1, 17.5 and, in 8, 18.9).  With more planes they never did
-// (100^3: 28.6, 31.3, 37.6 us; a symmetric 512^3: 958, 1277, 1680 us, where the
-// one-voxel sweep's tiles of 13 and 8 rows had taken 1162 and 1364), so the
-// hint is not followed there.
+// 12; 64^3 17.1, 17.5 and, in 8, 18.9), or where they take no more tiles and
+// leave fewer warps idle (512 x 8 x 512: 54.3 us in 20 rows, 49.7 in 12).  Else they
+// never did (100^3: 28.6, 31.3, 37.6 us; a symmetric 512^3: 958, 1277, 1680 us,
+// where the one-voxel sweep's tiles of 13 and 8 rows had taken 1162 and 1364),
+// so the hint is not followed.
 template <int MAXI>
 static int pair_rows(const Launch<float, MAXI>& L, int tile_y)
 {
     const int rows = tile_y == 8 ? 8 : tile_y == 13 ? 12 : 20;
-    return pair_units(L, 20) > 4LL * device_sms() ? 20 : rows;
+    const long long units = pair_units(L, 20);
+    return units <= 4LL * device_sms() || units == pair_units(L, rows) ? rows : 20;
 }
 
 template <int MAXI, bool SYM, bool HALO>
