@@ -73,19 +73,20 @@ typedef struct {
     double xi;              /* regularisation > 0 (Sec. 4.1; 1e-6 in the paper)          */
     double a[6];            /* a20 a11 a02 a10 a01 a00 of eq. F, kappa1 >= kappa2         */
     /* Tile height: 0 = automatic, else 8, 13 or 16.  FP32: a hint for gradients
-     * and steps of small launches (at most four planes of 20-row tiles per SM),
-     * where 8 selects 8 rows and 13 selects 12; every other FP32 launch, and 16,
-     * takes the automatic height (20 rows, or 28 for symmetric polynomials where
-     * that pads less; 24 or 30 for the energy alone).  FP64: the fused sweep with
-     * that many rows; a nonzero tile_y or tile_z also keeps grids of up to 2^22
-     * voxels off the two-kernel form that is automatic there and faster. */
+     * and steps of small launches (at most four planes of 20-row tiles per SM) and
+     * of grids that take no more of the smaller tiles, where 8 selects 8 rows and
+     * 13 selects 12; every other FP32 launch, and 16, takes the automatic height
+     * (20 rows, or 28 for symmetric polynomials where that pads less; 24 or 30
+     * for the energy alone).  FP64: the fused sweep with that many rows; a nonzero
+     * tile_y or tile_z also keeps grids of up to 2^22 voxels off the two-kernel
+     * form that is automatic there and faster. */
     int32_t tile_y;
     int32_t tile_z;         /* 0 = automatic; else planes per CTA z-chunk (>= 1)         */
     /* Orientation term of Sec. 5.2: eps mu (theta . grad u)^2 joins the
      * integrand (grad u the central-difference gradient).  mu = 0 (with any
      * theta) is the plain eq. Feps.  theta (x, y, z) is used as given; the
      * paper takes it of unit norm.  Fused path only (PFC_EUNSUPPORTED on the
-     * plain path and in batches); it runs the extended sweep (8-row tiles). */
+     * plain path and in batches); it runs the extended sweep. */
     double mu;
     double theta[3];
     /* 1: the tangent-projected M = -eps P Hess u P, P = I - n (x) n (the form
@@ -184,9 +185,10 @@ pfc_status pfc_surface_cells(pfc_ctx* ctx, const void* u, double level, void* ce
  * sums the areas of the cells whose kappa1 falls in bin b1 and kappa2 in bin
  * b2 of [lo, hi) split in nbins; values outside are clamped into the edge bins
  * (the paper truncates its diagrams to [-100, 100]).  FP64 atomics: the sums
- * are exact up to rounding order.  Enqueue only, on any stream; a call with
- * many cells takes up to 16 MB of scratch in the order of the stream, from a
- * pool of which the context keeps 32 MB (a captured call takes none). */
+ * are exact up to rounding order.  Enqueue only, on any stream: a call with
+ * many cells for its bins works in 16 MB of the context's memory, made by the
+ * first such call, and its stream waits for the last one on any stream; a
+ * captured call uses none of the context's memory. */
 pfc_status pfc_curvature_histogram(pfc_ctx* ctx, const void* cells, int64_t n, int32_t nbins, double lo,
                                    double hi, double* hist_dev, pfc_stream stream);
 

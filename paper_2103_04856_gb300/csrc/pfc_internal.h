@@ -218,8 +218,9 @@ cudaError_t launch_surface_count(const T* u, int nx, int ny, int nz, double leve
 template <typename T>
 cudaError_t launch_surface_cells(const T* u, const T* k1, const T* k2, int nx, int ny, int nz, double h, double level,
                                  unsigned* work, long long* offsets, T* cells, long long cap, cudaStream_t s);
-// part: histogram_copies(n, nbins) tables of nbins^2 values to work in, or
-// null: then hist itself
+// part: histogram_copies(n, nbins) tables of nbins^2 values to work in, at most
+// HIST_BYTES, or null: then hist itself
+constexpr size_t HIST_BYTES = 16u << 20;
 int histogram_copies(long long n, int nbins);
 template <typename T>
 cudaError_t launch_curvature_histogram(const T* cells, long long n, int nbins, double lo, double hi, double* part,

@@ -428,16 +428,16 @@ template cudaError_t launch_surface_cells<float>(const float*, const float*, con
 template cudaError_t launch_surface_cells<double>(const double*, const double*, const double*, int, int, int, double,
                                                   double, unsigned*, long long*, double*, long long, cudaStream_t);
 
-// Tables of the histogram: one per SM while they take no more than 16 MB.  Few
+// Tables of the histogram: one per SM while they take no more than HIST_BYTES.  Few
 // cells for the bins add into one: its atomics take about 10 ns times n / nbins
 // (20 to 700 bins of smooth surfaces; noise a little less above 100 bins), and
-// the tables' own scratch, clearing and sum make a call 24 us instead of 16.
+// the tables' clearing and sum make a call 24 us instead of 16.
 // 100 bins: 110 000 cells 18 us (24 in tables), 240 000 29 (25), 7.2 million 725 (69).
 int histogram_copies(long long n, int nbins)
 {
     if (n < 1600LL * nbins) return 1;
     const double bytes = 8.0 * nbins * nbins;
-    const double c = 16.0 * 1024 * 1024 / bytes;
+    const double c = HIST_BYTES / bytes;
     return c < 2.0 ? 1 : (c < device_sms() ? (int)c : device_sms());
 }
 
