@@ -83,8 +83,8 @@ __device__ __forceinline__ double rsq(double a) { return rsqrt(a); }
 
 // Coefficients of eq. Feps and the stencil scales as pairs, for the general
 // form, formed once per run (2 c2 is not: without its registers the batched
-// step spills 80/148 bytes a thread instead of 124/192, 24 mixed problems
-// 5.8 -> 5.5 ms for 16 steps).
+// step spills 92/144 bytes a thread, stores/loads, instead of 124/192, 24 mixed
+// problems 5.8 -> 5.5 ms for 16 steps).
 struct Coef2 {
     F2 c1, c2, c3, c4, c5, c6, c6x2, kd, ko, ko2, sg, nsg, ie, xi2;
     F2 c7, c7x2, th0, th1, th2;       // orientation term (ORIENT)

@@ -27,7 +27,8 @@
 // voxels (168 registers) hide less latency than twenty of one, so the square
 // root's softplus is branch-free (root_softplus) and the run bookkeeping lives
 // in shared memory (the general form spilled 240 bytes per thread with it in
-// registers).  Tiles of 20 rows (28 for symmetric polynomials, see sym_tall): 12 and 8 rows ran 1.17 and 1.6 times longer
+// registers; without, a single problem's 16 to 24, a batch's 92 and the a(x)
+// sweep's 104).  Tiles of 20 rows (28 for symmetric polynomials, see sym_tall): 12 and 8 rows ran 1.17 and 1.6 times longer
 // on a 512^3 field.  A phase per plane on an mbarrier, waited for two planes
 // later, instead of a barrier per plane was 19 % slower.
 // Against the one-voxel sweep before it (32 x 16 and 32 x 13 tiles): four
